@@ -245,8 +245,8 @@ class CpWorkload:
         sm_mhz = float(measured_peaks().get("sm_max_mhz", 2070.0))
         peak = props.multi_processor_count * 128 * 2 * sm_mhz * 1e6 / 1e12
         ach = self.flops() / (t / 1e3) / 1e12
-        files = ["fcs_cp.cu", "fcs_cp_run.cuh", "fcs_fft.cuh", "fcs_hash.cuh", "fcs_internal.cuh"]
-        return {"kernel": "cp13_kernel (fcs_sketch_cp_seeded: prep launch with the hash "
+        files = ["fcs_cp.cu", "fcs_cp_run.cuh", "fcs_pair.cuh", "fcs_fft.cuh", "fcs_hash.cuh", "fcs_internal.cuh"]
+        return {"kernel": "cp_pair_kernel (fcs_sketch_cp_seeded: prep launch with the hash "
                           "tables + fused sketch)",
                 "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak,
@@ -626,11 +626,12 @@ class BatchWorkload:
         return sum(D for _, _, _, D in self.shapes)
 
     def launches_per_step(self):
-        # batched transpose + one kernel per FFT size; problems with
-        # P > 16384 run on the two-pass long-FFT route after them
-        sizes = {fft_len(jt_of(J)) for _, J, _, _ in self.shapes if fft_len(jt_of(J)) <= 16384}
+        # batched transpose + one kernel per FFT size (at least: a size whose
+        # longest hash ranges need more shared memory takes two); problems
+        # with P > 32768 run on the two-pass long-FFT route after them
+        sizes = {fft_len(jt_of(J)) for _, J, _, _ in self.shapes if fft_len(jt_of(J)) <= 32768}
         return 1 + len(sizes) + sum(long_cp_launches(J) for _, J, _, _ in self.shapes
-                                    if fft_len(jt_of(J)) > 16384)
+                                    if fft_len(jt_of(J)) > 32768)
 
     def setup(self, fcs, ctx, dev):
         import torch
@@ -747,7 +748,7 @@ class BatchWorkload:
                 "peak_source": f"derived: {props.multi_processor_count} SMs x 128 FP32 lanes "
                                f"x 2 flop/FMA x {sm_mhz:.0f} MHz",
                 "avg_launch_ms": t, "grain": self.grain,
-                "classes": [{"fft_len": P, "engine": "warp-DIT" if e else "slot FFT",
+                "classes": [{"fft_len": P, "engine": "row-pair" if e else "slot FFT",
                              "thread_mult": m, "items_per_cta": i, "threads": n}
                             for P, m, i, n, e in self.plan.config()[1]],
                 "plain_per_problem_ms": plain_ms,

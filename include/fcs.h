@@ -33,14 +33,14 @@
  *    FFT-based calls (CP route, contractions, outer combine) need
  *    Jt <= 2^20: the FFT length is P = smallest power of
  *    two >= Jt, 16 <= P <= 2^20, else FCS_EUNSUPPORTED.  P <= 16384 runs one
- *    transform per CTA in shared memory.  The CP route at P = 32768 runs one
- *    fused kernel (one 2^14-point transform per CTA in shared memory, a
- *    128 KiB running-product slice per CTA in the context workspace, fewer
- *    CTAs when the budget is small).  Other longer transforms use a two-pass
+ *    transform per CTA in shared memory, and so does the CP route at
+ *    P = 32768 with every J_n <= 17984 (with a longer one it keeps a 128 KiB
+ *    running-product slice per CTA in the context workspace, with fewer CTAs
+ *    when the budget is small).  Other longer transforms use a two-pass
  *    FFT through the context workspace (at most min(budget, 512 MiB), work
  *    split into chunks that fit; a few MiB suffice).  fcs_sketch_cp_noalloc
- *    takes P <= 16384.  Batch plans run P <= 16384 in their per-FFT-size
- *    launch chain and longer problems with the launches above.
+ *    takes P <= 16384.  Batch plans run P <= 32768 in their per-FFT-size
+ *    launch chain and other problems with the launches above.
  *  - The library allocates only its own context workspace (device memory
  *    reused across calls, bounded by the context's budget), a 256 KiB
  *    twiddle table, the staging buffer of fcs_sketch_cp_host when that is
@@ -155,9 +155,11 @@ int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
  *   Workspace for P <= 16384: A + 256 + 4*R*sum_n(I_n) bytes, rounded up to
  *   a multiple of 256, with A = D*(P/2+2)*8 rounded up to a multiple of 256
  *   (spectrum accumulator, tickets, factor columns transposed with lambda
- *   folded in).  P = 32768: A + 256 + 128 KiB per CTA (fewer CTAs, down to
- *   one, when the budget is smaller).  Longer: the two-pass route, chunked to
- *   what the budget allows (a few MiB suffice).
+ *   folded in).  P = 32768 with every J_n <= 17984: the same, or A + 256 bytes
+ *   (factors read in place) when that exceeds min(budget, 512 MiB); with a
+ *   longer J_n: A + 256 + 128 KiB per CTA (fewer CTAs, down to one, when the
+ *   budget is smaller).  Longer: the two-pass route, chunked to what the
+ *   budget allows (a few MiB suffice).
  */
 int fcs_sketch_cp(fcs_ctx *ctx, int N, const int64_t *host_I,
                   const int32_t *host_J, int64_t R, int D,
@@ -173,7 +175,8 @@ int fcs_sketch_cp(fcs_ctx *ctx, int N, const int64_t *host_I,
  * sketch of [[lambda; U_1..U_N]] to out [D][Jt], as fcs_sketch_cp with
  * those tables.  For P <= 16384 the tables are written by the same launch
  * that transposes the factors, so the call issues two kernels instead of
- * three; longer transforms generate them with their own launch first.
+ * three; so they are at P = 32768 when the factors are transposed, and other
+ * long transforms generate them with their own launch first.
  * Arguments, workspace and errors otherwise as fcs_sketch_cp (and I_n <= 2^32
  * as fcs_make_hashes).
  */
@@ -243,12 +246,15 @@ int fcs_sketch_cp_noalloc(void *stream, int N, const int64_t *host_I,
  * order, sizes, rank and sketch length run in a few launches: the work is
  * cut into items (problem, sketch d, group of `grain` ranks) and grouped by
  * FFT length; one batched launch transposes every problem's factor columns,
- * then one kernel per FFT length P <= 16384 runs its items (one CTA per
- * item, largest FFT first), the kernels chained by programmatic dependent
- * launch so that each starts while the previous one drains.  The item that
- * completes a sketch (a ticket counter) runs its inverse FFT.  Problems with
- * P > 16384 follow with the long-FFT launches of fcs_sketch_cp, from
- * plan-owned scratch.  Results equal fcs_sketch_cp on each problem up to
+ * then one kernel per FFT length P <= 32768 runs its items (one CTA per
+ * item, largest FFT first; two kernels where the longest hash ranges of a
+ * length take more shared memory), the kernels chained by programmatic
+ * dependent launch so that each starts while the previous one drains.  The
+ * item that completes a sketch (a ticket counter) runs its inverse FFT.
+ * Problems with P > 32768, or with P = 32768 and a J_n > 17984, follow with
+ * the long-FFT launches of fcs_sketch_cp, from plan-owned scratch; so do the
+ * other problems at P = 32768 when the plan would exceed the budget with
+ * them in the chain.  Results equal fcs_sketch_cp on each problem up to
  * FP32 summation order.
  */
 typedef struct fcs_cp_problem {
@@ -271,8 +277,8 @@ typedef struct fcs_batch_plan fcs_batch_plan;
 /* Validate a batch, cut its items and upload descriptors into plan-owned
  * device memory (counted against the context budget).  grain = ranks per
  * item; 0 = the autotuned grain for this batch shape if fcs_batch_autotune
- * has seen it (this context or the FCS_AUTOTUNE_CACHE file), else a default
- * of about four items per SM.  The class shapes are the autotuned ones for
+ * has seen it (this context or the FCS_AUTOTUNE_CACHE file), else chosen
+ * problem by problem, for items of about equal length within an FFT length.  The class shapes are the autotuned ones for
  * this batch shape when known, else the defaults.  The plan records the problems' device
  * pointers: later launches read whatever those buffers hold then. */
 int fcs_batch_plan_create(fcs_ctx *ctx, int nprob, const fcs_cp_problem *host_probs,
@@ -292,9 +298,10 @@ int fcs_batch_sketch_cp(fcs_ctx *ctx, int nprob, const fcs_cp_problem *host_prob
                         int grain);
 
 /* Shape of one FFT-length class of a batch plan.  engine: 0 = the slot FFT
- * (Stockham passes in shared memory, P <= 8192), 1 = the warp-DIT engine
- * (512-point sub-FFTs per warp, then a column step per thread; P = 8192, where
- * it is the default, and P = 16384, the only engine there).  thread_mult (slot FFT only): 1 = one
+ * (Stockham passes in shared memory, P <= 8192), 1 = the row-pair engine
+ * (512-point sub-FFTs, two at a time per warp, then a column step per thread;
+ * P = 8192, where it is the default, and P = 16384, the only engine there;
+ * P = 32768 has one shape and is not listed).  thread_mult (slot FFT only): 1 = one
  * radix-16 butterfly per thread (P/32 threads, at least 32), 2 = twice as
  * many threads.  items_per_cta: 1, 2 or 4 work items run one after another by
  * each CTA.  threads: the block size that results (output of
@@ -308,19 +315,20 @@ typedef struct fcs_batch_class_cfg {
 } fcs_batch_class_cfg;
 
 /* fcs_batch_plan_create with explicit class shapes (classes not listed take
- * the warp-DIT engine at P = 8192 and 16384, the slot FFT below, with
+ * the row-pair engine at P = 8192 and 16384, the slot FFT below, with
  * thread_mult = 1 and items_per_cta = 1) and grain (0 = the default grain). */
 int fcs_batch_plan_create_cfg(fcs_ctx *ctx, int nprob, const fcs_cp_problem *host_probs,
                               int grain, int ncfg, const fcs_batch_class_cfg *host_cfg,
                               fcs_batch_plan **plan);
 
-/* The grain and class shapes a plan was built with: *host_ncfg classes (the
+/* The grain (0: chosen problem by problem) and class shapes a plan was built
+ * with: *host_ncfg classes (the
  * first max_cfg of them copied to host_cfg, largest FFT first). */
 int fcs_batch_plan_config(const fcs_batch_plan *plan, int *host_grain, int max_cfg,
                           fcs_batch_class_cfg *host_cfg, int *host_ncfg);
 
 /* Autotuner: times the whole batch on the device.  First the grain (ranks
- * per item: 1, 2, 4, ... up to 64 and 2R) with every class at its default
+ * per item: 0, i.e. problem by problem, 1, 2, 4, ... up to 64 and 2R) with every class at its default
  * shape; then, class by class from the largest FFT, every engine (for
  * P = 8192), thread_mult and items_per_cta with the other classes at their
  * best so far, a shape replacing the current one only when at least 3 %

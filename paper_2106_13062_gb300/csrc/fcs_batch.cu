@@ -66,42 +66,52 @@ struct TransposeTask {
   int64_t tiles_i, tile0;   // tiles along I; first flat tile index
 };
 
-// One CTA per 32x32 tile of one factor matrix; the task is found by binary
-// search over the tasks' first tile indices.
-__global__ void batch_transpose_kernel(const TransposeTask *__restrict__ tasks, int ntasks) {
-  __shared__ float tile[32][33];
+// One CTA per tile of kTI rows by 32 columns of one factor matrix.  The task
+// is the last one whose first tile is not beyond this one: every thread looks
+// at tasks of its own, so finding it costs one memory latency (a binary
+// search over 230 tasks costs eight, as long as the copy of a 32 x 32 tile).
+constexpr int kTI = 128;
+__global__ void __launch_bounds__(256) batch_transpose_kernel(const TransposeTask *__restrict__ tasks,
+                                                              int ntasks) {
+  __shared__ float tile[kTI][33];
+  __shared__ int mine;
   const int64_t t = blockIdx.x;
-  int lo = 0, hi = ntasks - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) / 2;
-    if (tasks[mid].tile0 <= t) lo = mid; else hi = mid - 1;
-  }
-  const TransposeTask T = tasks[lo];
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  for (int k = tid; k < ntasks; k += 256)
+    if (tasks[k].tile0 <= t && (k + 1 == ntasks || tasks[k + 1].tile0 > t)) mine = k;
+  __syncthreads();
+  const TransposeTask T = tasks[mine];
   const int64_t local = t - T.tile0;
-  const int64_t i0 = (local % T.tiles_i) * 32, r0 = (local / T.tiles_i) * 32;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int64_t i = i0 + k, r = r0 + threadIdx.x;
-    if (i < T.I && r < T.R) tile[k][threadIdx.x] = T.U[i * T.ld + r];
+  const int64_t i0 = (local % T.tiles_i) * kTI, r0 = (local / T.tiles_i) * 32;
+  const int64_t r = r0 + threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < kTI; k += 8) {
+    const int64_t i = i0 + k + threadIdx.y;
+    if (i < T.I && r < T.R) tile[k + threadIdx.y][threadIdx.x] = T.U[i * T.ld + r];
   }
   __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int64_t r = r0 + k, i = i0 + threadIdx.x;
-    if (i < T.I && r < T.R) {
-      const float lam = T.lambda ? __ldg(T.lambda + r) : 1.f;
-      T.UT[r * T.I + i] = tile[threadIdx.x][k] * lam;
+#pragma unroll
+  for (int k = threadIdx.y; k < 32; k += 8) {
+    const int64_t q = r0 + k;
+    if (q >= T.R) break;
+    const float lam = T.lambda ? __ldg(T.lambda + q) : 1.f;
+#pragma unroll
+    for (int j = 0; j < kTI; j += 32) {
+      const int64_t i = i0 + j + threadIdx.x;
+      if (i < T.I) T.UT[q * T.I + i] = tile[j + threadIdx.x][k] * lam;
     }
   }
 }
 
-// Engine of a class without a tuned or explicit shape: the warp-DIT engines
-// where they exist (P = 8192 and 16384), the slot FFT below.
-int default_engine(int L) { return (L == wdit::kL || L == 12) ? 1 : 0; }
+// Engine of a class without a tuned or explicit shape: the row-pair engine
+// where it exists (P = 8192 .. 32768), the slot FFT below.
+int default_engine(int L) { return L >= 12 ? 1 : 0; }
 
 // Class kernel for log2 M = L with engine eng, at thread multiplier ntm (slot
-// FFT only; the warp-DIT engines have one thread count) running ipc items
+// FFT only; the row-pair engine has one thread count) running ipc items
 // per CTA.
 ClassKernel class_kernel(int L, int eng, int ntm, int ipc, int64_t Imax, int sb) {
-  if (L == wdit::kL) return class_kernel_13(ipc, Imax, sb);
+  if (L >= 13) return class_kernel_13(L, ipc, sb);
   if (L == 12) return class_kernel_12(eng, ntm, ipc, Imax, sb);
   if (L >= 10) return class_kernel_mid(L, ntm, ipc, Imax, sb);
   return class_kernel_small(L, ntm, ipc, Imax, sb);
@@ -109,12 +119,23 @@ ClassKernel class_kernel(int L, int eng, int ntm, int ipc, int64_t Imax, int sb)
 
 size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// The longest scatter buffer (floats) with which as many blocks of the
+// row-pair engine share an SM as its registers allow.
+template <int NR>
+constexpr int pair_full_sb() {
+  return int((233472 / pfft::Geo<NR>::CTAS - 1024 - 256 - pfft::Smem<NR>::bytes(0)) /
+             (sizeof(float4) * (NR / 2))) *
+         2 * NR;
+}
+
 // Per-problem facts derived on the host.
 struct HostProb {
   Modes m;
   int L, sb;
   int64_t R, utlen, Imax;
-  bool longp;                  // P > 16384: not for the batch kernels
+  int tall;                    // 1: its scatter buffer costs the row-pair engine a resident block
+  bool longp;                  // not for the batch kernels: P > 32768, or 32768 with a hash
+                               // range beyond the row-pair engine's scatter buffer
 };
 
 int check_problem(fcs_ctx *ctx, int k, const fcs_cp_problem &q, HostProb *hp) {
@@ -136,9 +157,10 @@ int check_problem(fcs_ctx *ctx, int k, const fcs_cp_problem &q, HostProb *hp) {
   if (log2p > kMaxLog2PBig)
     return set_error(ctx, FCS_EUNSUPPORTED, "problem %d: Jt=%lld needs FFT length > %d", k,
                      (long long)hp->m.Jt, 1 << kMaxLog2PBig);
-  hp->longp = log2p > kMaxLog2P;
+  hp->longp = log2p > kMaxLog2P + 1 || (log2p == kMaxLog2P + 1 && jmax > kPair32MaxJ);
   hp->L = log2p - 1;
   hp->sb = int((jmax + 3) / 4 * 4);
+  hp->tall = hp->L == 12 ? hp->sb > pair_full_sb<8>() : hp->L == 13 ? hp->sb > pair_full_sb<16>() : 0;
   hp->R = q.R;
   hp->utlen = ut;
   hp->Imax = imax;
@@ -207,18 +229,61 @@ void save_cache(const fcs_batch_state &st) {
   fclose(f);
 }
 
-int default_grain(const fcs_ctx *ctx, int nprob, const fcs_cp_problem *q) {
-  int64_t work = 0;
-  int64_t rmax = 1;
-  for (int k = 0; k < nprob; ++k) {
-    work += int64_t(q[k].D) * q[k].R;
-    rmax = std::max<int64_t>(rmax, q[k].R);
+// The shape of the FFT-size class L (defaults where cfg names none).
+ClassCfg class_cfg(int L, const std::vector<ClassCfg> *cfg) {
+  ClassCfg c{L, 1, 1, default_engine(L)};
+  if (cfg)
+    for (const ClassCfg &x : *cfg)
+      if (x.L == L) c = x;
+  c.eng = L >= 13 ? 1 : (L == 12 && c.eng == 1 ? 1 : 0);
+  if (c.eng == 1 || (c.ntm != 1 && c.ntm != 2)) c.ntm = 1;
+  if (c.ipc != 1 && c.ipc != 2 && c.ipc != 4) c.ipc = 1;
+  return c;
+}
+
+// Ranks per item, problem by problem, when the caller names no grain.  Every
+// item of an FFT-size class is to take about the same time, in transforms:
+// a quarter of what one resident block gets of the class, so that the last
+// items of a class leave a resident block idle for an eighth of it at most on
+// average, but at least 8 transforms, since starting an item and publishing
+// its spectrum cost about as much as one.  A class with less work than that
+// takes as many items as there are resident blocks.  (One grain for all,
+// about four items per SM, gave the 64-problem mix items of up to 64
+// transforms and 3.4 waves of them at P = 16384.)
+std::vector<int64_t> balanced_ranks(fcs_ctx *ctx, const std::vector<HostProb> &hp, int nprob,
+                                    const fcs_cp_problem *q, const std::vector<ClassCfg> *cfg) {
+  std::map<int, double> per_item;         // by launch: 2 L + tall
+  auto key = [&](int k) { return 2 * hp[k].L + hp[k].tall; };
+  for (int k = 0; k < nprob; ++k) per_item[key(k)] += double(q[k].D) * double(hp[k].R) * q[k].N;
+  for (auto &c : per_item) {
+    int64_t Imax = 1;
+    int sb = 4;
+    for (int k = 0; k < nprob; ++k)
+      if (key(k) == c.first) {
+        Imax = std::max(Imax, hp[k].Imax);
+        sb = std::max(sb, hp[k].sb);
+      }
+    const ClassCfg cc = class_cfg(c.first / 2, cfg);
+    const ClassKernel ck = class_kernel(c.first / 2, cc.eng, cc.ntm, cc.ipc, Imax, sb);
+    int per_sm = ck.per_sm;
+    if (per_sm == 0 &&
+        (!ck.fn || allow_smem(ck.fn, ck.smem) != cudaSuccess ||
+         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ck.fn, ck.nt, ck.smem) !=
+             cudaSuccess)) {
+      cudaGetLastError();
+      per_sm = 1;
+    }
+    if (per_sm < 1) per_sm = 1;
+    const double each = c.second / (double(std::max(1, ctx->sm_count)) * per_sm);
+    c.second = each <= 8. ? each : std::max(8., each / 4.);
   }
-  // about four items per SM, power-of-two grain
-  int64_t g = work / (4 * int64_t(std::max(1, ctx->sm_count)));
-  int grain = 1;
-  while (grain * 2 <= g && grain < 64) grain *= 2;
-  return int(std::min<int64_t>(grain, rmax));
+  std::vector<int64_t> r(nprob);
+  for (int k = 0; k < nprob; ++k) {
+    const int64_t want = std::max<int64_t>(1, int64_t(per_item[key(k)] / q[k].N + 0.5));
+    const int64_t groups = (hp[k].R + want - 1) / want;
+    r[k] = (hp[k].R + groups - 1) / groups;
+  }
+  return r;
 }
 
 }  // namespace
@@ -238,15 +303,17 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
     if (rc) return rc;
     if (hp[k].longp)
       return set_error(ctx, FCS_EUNSUPPORTED,
-                       "problem %d: FFT length > %d is not run by the batch kernels", k,
-                       1 << kMaxLog2P);
+                       "problem %d: FFT length %d is not run by the batch kernels", k,
+                       2 << hp[k].L);
   }
   std::vector<int4> items;
   std::vector<BatchProb> probs(nprob);
   int ntask = 0;
   size_t g_bytes = 0, t_count = 0, ut_len = 0;
+  const std::vector<int64_t> even = grain < 1 ? balanced_ranks(ctx, hp, nprob, q, cfg)
+                                              : std::vector<int64_t>();
   for (int k = 0; k < nprob; ++k) {
-    const int64_t rpi = std::min<int64_t>(std::max(grain, 1), hp[k].R);
+    const int64_t rpi = grain < 1 ? even[k] : std::min<int64_t>(grain, hp[k].R);
     const int groups = int((hp[k].R + rpi - 1) / rpi);
     memset(&probs[k], 0, sizeof(BatchProb));
     probs[k].rpi = rpi;
@@ -258,9 +325,10 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
     ut_len += size_t(hp[k].utlen);
     ntask += q[k].N;
   }
-  // largest FFT first, then the longest items (ranks x modes)
+  // largest FFT first, within a size the tall scatter buffers, then the
+  // longest items (ranks x modes)
   std::stable_sort(items.begin(), items.end(), [&](const int4 &x, const int4 &y) {
-    const int lx = hp[x.x].L, ly = hp[y.x].L;
+    const int lx = 2 * hp[x.x].L + hp[x.x].tall, ly = 2 * hp[y.x].L + hp[y.x].tall;
     if (lx != ly) return lx > ly;
     return probs[x.x].rpi * q[x.x].N > probs[y.x].rpi * q[y.x].N;
   });
@@ -298,6 +366,7 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
     for (int n = 0; n < kMaxN; ++n) {
       P.I[n] = hp[k].m.I[n];
       P.off[n] = hp[k].m.off[n];
+      P.J[n] = hp[k].m.J[n];
     }
     P.ldh = hp[k].m.ldh;
     P.Jt = hp[k].m.Jt;
@@ -319,7 +388,7 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
       T.I = q[k].I[n];
       T.R = P.R;
       T.ld = q[k].ldU[n];
-      T.tiles_i = (T.I + 31) / 32;
+      T.tiles_i = (T.I + kTI - 1) / kTI;
       T.tile0 = tiles;
       tiles += T.tiles_i * ((T.R + 31) / 32);
       tasks.push_back(T);
@@ -330,28 +399,19 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
   // one launch per FFT-size class: prefetch depth and scatter buffer sized
   // for the class's largest problem
   for (size_t i = 0; i < items.size();) {
-    const int L = hp[items[i].x].L;
+    const int L = hp[items[i].x].L, tall = hp[items[i].x].tall;
     size_t j = i;
     int64_t Imax = 0;
     int sb = 4;
-    for (; j < items.size() && hp[items[j].x].L == L; ++j) {
+    for (; j < items.size() && hp[items[j].x].L == L && hp[items[j].x].tall == tall; ++j) {
       Imax = std::max(Imax, hp[items[j].x].Imax);
       sb = std::max(sb, hp[items[j].x].sb);
     }
-    ClassCfg c{L, 1, 1, default_engine(L)};
-    if (cfg)
-      for (const ClassCfg &x : *cfg)
-        if (x.L == L) c = x;
-    c.eng = L == wdit::kL ? 1 : (L == 12 && c.eng == 1 ? 1 : 0);
-    if (c.eng == 1 || (c.ntm != 1 && c.ntm != 2)) c.ntm = 1;
-    if (c.ipc != 1 && c.ipc != 2 && c.ipc != 4) c.ipc = 1;
+    const ClassCfg c = class_cfg(L, cfg);
     const ClassKernel ck = class_kernel(L, c.eng, c.ntm, c.ipc, Imax, sb);
     if (!ck.fn) return set_error(ctx, FCS_EUNSUPPORTED, "no batch kernel for log2 M = %d", L);
-    if (ck.smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(ck.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           int(ck.smem));
-      if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(batch class)");
-    }
+    const cudaError_t e = allow_smem(ck.fn, ck.smem);
+    if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(batch class)");
     bb.classes.push_back(
         BatchClass{ck.fn, ck.nt, ck.smem, int(i), int(j - i), L, c.ntm, c.ipc, c.eng});
     i = j;
@@ -402,10 +462,6 @@ int batch_issue(fcs_ctx *ctx, char *base, const BatchBuild &b) {
   return FCS_OK;
 }
 
-int batch_default_grain(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q) {
-  return default_grain(ctx, nprob, q);
-}
-
 namespace {
 
 // Build a plan: lay the batch out in plan-owned device memory and upload the
@@ -413,21 +469,44 @@ namespace {
 int plan_create(fcs_ctx *ctx, int nprob_all, const fcs_cp_problem *q_all, int grain,
                 fcs_batch_plan **out, const std::vector<ClassCfg> *cfg = nullptr) {
   *out = nullptr;
-  // problems with P > 16384 run after the batch kernels, each with the
-  // multi-kernel long-FFT route
+  // problems the batch kernels do not run follow them, one after another;
+  // P = 32768 joins those when the plan would not fit the budget otherwise
+  // (read in place there, without a transposed copy of the factors)
   std::vector<fcs_cp_problem> shortp, longp;
-  for (int k = 0; k < nprob_all; ++k) {
-    HostProb hp{};
-    int rc = check_problem(ctx, k, q_all[k], &hp);
-    if (rc) return rc;
-    (hp.longp ? longp : shortp).push_back(q_all[k]);
+  BatchBuild bb{};
+  std::vector<char> desc;
+  int rc = FCS_OK;
+  size_t long_need = 0, long_cap = 0;
+  for (int top : {kMaxLog2P, kMaxLog2P - 1}) {
+    shortp.clear();
+    longp.clear();
+    for (int k = 0; k < nprob_all; ++k) {
+      HostProb hp{};
+      rc = check_problem(ctx, k, q_all[k], &hp);
+      if (rc) return rc;
+      (hp.longp || hp.L > top ? longp : shortp).push_back(q_all[k]);
+    }
+    bb = BatchBuild{};
+    if (!shortp.empty()) {
+      rc = batch_build(ctx, int(shortp.size()), shortp.data(), grain, nullptr, &desc, &bb, cfg);
+      if (rc) return rc;
+    }
+    // scratch for the long problems, run one after another; a modest cap
+    // keeps the plan small (their routes work in chunks)
+    const size_t held = ctx->ws_bytes + ctx->plan_bytes + bb.total;
+    const size_t room = ctx->budget > held ? ctx->budget - held : 0;
+    long_cap = std::min<size_t>(room, size_t(256) << 20);
+    long_need = 0;
+    for (const fcs_cp_problem &p : longp) {
+      Modes m{};
+      make_modes(ctx, p.N, p.I, p.J, p.ldh, &m);
+      long_need = std::max(long_need, big_sketch_cp_bytes(m, p.R, p.D, ilog2_ceil(m.Jt), long_cap,
+                                                          ctx->sm_count));
+    }
+    if (held <= ctx->budget && long_need <= long_cap) break;
   }
   const int nprob = int(shortp.size());
   const fcs_cp_problem *q = shortp.data();
-  BatchBuild bb{};
-  std::vector<char> desc;
-  int rc = nprob ? batch_build(ctx, nprob, q, grain, nullptr, &desc, &bb, cfg) : FCS_OK;
-  if (rc) return rc;
   if (ctx->ws_bytes + ctx->plan_bytes + bb.total > ctx->budget)
     return set_error(ctx, FCS_ENOMEM_BUDGET,
                      "batch plan of %zu bytes exceeds the context budget of %zu", bb.total,
@@ -457,28 +536,16 @@ int plan_create(fcs_ctx *ctx, int nprob_all, const fcs_cp_problem *q_all, int gr
   plan->owner = ctx;
   plan->longp = longp;
   if (!longp.empty()) {
-    // one scratch buffer for the long problems, run one after another; a
-    // modest cap keeps the plan small (the route works in chunks)
-    size_t room = ctx->budget > ctx->ws_bytes + ctx->plan_bytes + bb.total
-                      ? ctx->budget - (ctx->ws_bytes + ctx->plan_bytes + bb.total)
-                      : 0;
-    const size_t cap = std::min<size_t>(room, size_t(256) << 20);
-    size_t need = 0;
-    for (const fcs_cp_problem &p : longp) {
-      Modes m{};
-      make_modes(ctx, p.N, p.I, p.J, p.ldh, &m);
-      const int log2p = ilog2_ceil(m.Jt);
-      need = std::max(need, big_sketch_cp_bytes(m, p.R, p.D, log2p, cap, ctx->sm_count));
-    }
-    cudaError_t e = need > cap ? cudaErrorMemoryAllocation : cudaMalloc(&plan->long_ws, need);
+    cudaError_t e = long_need > long_cap ? cudaErrorMemoryAllocation
+                                         : cudaMalloc(&plan->long_ws, long_need);
     if (e != cudaSuccess) {
       cudaGetLastError();
       if (plan->dev) cudaFree(plan->dev);
       delete plan;
       return set_error(ctx, FCS_ENOMEM_BUDGET, "no room for the long problems' scratch (%zu B)",
-                       need);
+                       long_need);
     }
-    plan->long_bytes = need;
+    plan->long_bytes = long_need;
   }
   for (int k = 0; k < nprob_all; ++k) {
     int64_t jt = 1;
@@ -497,29 +564,16 @@ int plan_create(fcs_ctx *ctx, int nprob_all, const fcs_cp_problem *q_all, int gr
 int plan_launch(fcs_ctx *ctx, const fcs_batch_plan *plan) {
   if (ctx->spec_cache)
     for (const auto &o : plan->outs) spec_cache_invalidate(ctx, o.first, o.second);
-  // The first long problem on the P = 2^15 warp-DIT route has its accumulator
-  // cleared before the chain and its kernel launched as a programmatic
-  // dependent of the chain's last class, so its CTAs take the SMs the chain
-  // frees while it drains.  The other long problems share the scratch and
-  // run one after another afterwards.
-  bool split = false;
-  auto long_call = [&](const fcs_cp_problem &p, int stage, bool *sp) -> int {
-    Modes m{};
-    int rc = make_modes(ctx, p.N, p.I, p.J, p.ldh, &m);
-    if (rc) return rc;
-    return big_sketch_cp(ctx, m, p.R, p.D, p.U, p.ldU, p.lambda, p.h, p.s, p.out,
-                         ilog2_ceil(m.Jt), plan->long_ws, plan->long_bytes, stage, sp);
-  };
-  if (plan->dev && !plan->longp.empty()) {
-    int rc = long_call(plan->longp[0], 1, &split);
-    if (rc) return rc;
-  }
   if (plan->dev) {
     int rc = batch_issue(ctx, static_cast<char *>(plan->dev), plan->build);
     if (rc) return rc;
   }
-  for (size_t k = 0; k < plan->longp.size(); ++k) {
-    int rc = long_call(plan->longp[k], k == 0 && split ? 2 : 0, nullptr);
+  for (const fcs_cp_problem &p : plan->longp) {
+    Modes m{};
+    int rc = make_modes(ctx, p.N, p.I, p.J, p.ldh, &m);
+    if (rc) return rc;
+    rc = big_sketch_cp(ctx, m, p.R, p.D, p.U, p.ldU, p.lambda, p.h, p.s, p.out,
+                       ilog2_ceil(m.Jt), plan->long_ws, plan->long_bytes);
     if (rc) return rc;
   }
   return FCS_OK;
@@ -602,7 +656,7 @@ extern "C" int fcs_batch_plan_create(fcs_ctx *ctx, int nprob, const fcs_cp_probl
   DeviceGuard g(ctx->device);
   // the autotuned shape of this batch (grain and class shapes), if any
   const auto *t = tuned_entry(ctx, nprob, host_probs);
-  if (grain < 1) grain = t ? t->first : default_grain(ctx, nprob, host_probs);
+  if (grain < 1) grain = t ? t->first : 0;
   return plan_create(ctx, nprob, host_probs, grain, plan, t ? &t->second : nullptr);
 }
 
@@ -622,7 +676,7 @@ extern "C" int fcs_batch_plan_create_cfg(fcs_ctx *ctx, int nprob,
     if (x.fft_len < 16 || x.fft_len > (1 << kMaxLog2P) || (x.fft_len & (x.fft_len - 1)))
       return set_error(ctx, FCS_EINVAL, "class %d: fft_len %d is not a power of two in [16, %d]",
                        c, x.fft_len, 1 << kMaxLog2P);
-    const int eng_ok = L == wdit::kL ? x.engine == 1 : L == 12 ? (x.engine == 0 || x.engine == 1)
+    const int eng_ok = L == 13 ? x.engine == 1 : L == 12 ? (x.engine == 0 || x.engine == 1)
                                                                : x.engine == 0;
     if (!eng_ok)
       return set_error(ctx, FCS_EINVAL, "class %d: engine %d not available for P = %d", c,
@@ -638,14 +692,17 @@ extern "C" int fcs_batch_plan_create_cfg(fcs_ctx *ctx, int nprob,
   int rc = ensure_batch_state(ctx);
   if (rc) return rc;
   DeviceGuard g(ctx->device);
-  if (grain < 1) grain = default_grain(ctx, nprob, host_probs);
+  if (grain < 1) grain = 0;
   return plan_create(ctx, nprob, host_probs, grain, plan, &cfg);
 }
 
 extern "C" int fcs_batch_plan_config(const fcs_batch_plan *plan, int *host_grain, int max_cfg,
                                      fcs_batch_class_cfg *host_cfg, int *host_ncfg) {
   if (!plan || !host_ncfg || (max_cfg > 0 && !host_cfg)) return FCS_EINVAL;
-  const auto &cls = plan->build.classes;
+  // (P = 32768 has one shape and cannot be named in a class list)
+  std::vector<BatchClass> cls;
+  for (const BatchClass &c : plan->build.classes)
+    if (c.L <= 13 && (cls.empty() || cls.back().L != c.L)) cls.push_back(c);
   *host_ncfg = int(cls.size());
   if (host_grain) *host_grain = plan->grain;
   for (int c = 0; c < int(cls.size()) && c < max_cfg; ++c)
@@ -713,12 +770,14 @@ extern "C" int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem 
     plan_free(plan);
     return r;
   };
-  // 1. ranks per item, every class at its default shape
+  // 1. ranks per item (0: chosen problem by problem), every class at its
+  //    default shape
   std::vector<ClassCfg> cfg;
   for (int L : sizes) cfg.push_back(ClassCfg{L, 1, 1, default_engine(L)});
-  int best = 1;
+  int best = 0;
   float best_ms = 1e30f;
-  for (int grain = 1; grain <= 64 && grain < 2 * rmax && rc == FCS_OK; grain *= 2) {
+  for (int grain = 0; grain <= 64 && grain < 2 * rmax && rc == FCS_OK;
+       grain = grain ? 2 * grain : 1) {
     float ms = 0.f;
     rc = timed(grain, cfg, &ms);
     if (rc == FCS_OK && ms < best_ms) {
@@ -733,9 +792,9 @@ extern "C" int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem 
     const ClassCfg keep = *c;
     ClassCfg bestc = keep;
     // shapes (engine, threads): slot FFT at 1 or 2 x the threads; for
-    // P = 8192 also the warp-DIT engine; P = 16384 has only warp-DIT
+    // P = 8192 also the row-pair engine, the only one beyond
     std::vector<std::pair<int, int>> shapes;
-    if (c->L == wdit::kL) {
+    if (c->L >= 13) {
       shapes = {{1, 1}};
     } else {
       shapes = {{0, 1}, {0, 2}};

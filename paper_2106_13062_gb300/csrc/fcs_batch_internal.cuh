@@ -9,13 +9,13 @@
 namespace fcs {
 
 // Tunable shape of one FFT-size class (log2 M = L): the engine (for P = 8192
-// the slot FFT or the warp-DIT engine; P = 16384 always runs warp-DIT, the
+// the slot FFT or the row-pair engine; beyond, always the row-pair engine, the
 // other sizes the slot FFT), the slot FFT's thread multiplier ntm (1 or 2:
 // M/16 or M/8 threads, at least a warp) and items run one after another per
 // CTA (ipc: 1, 2 or 4).
 struct ClassCfg {
   int L, ntm, ipc;
-  int eng = 0;               // P = 8192: 0 = slot FFT, 1 = warp-DIT engine
+  int eng = 0;               // P = 8192: 0 = slot FFT, 1 = row-pair engine
 };
 
 // One launch of a batch: the items [first, first + count) of one FFT size.
@@ -39,6 +39,7 @@ struct BatchBuild {
 };
 
 // Lay the batch out at device address `base` (NULL: sizes only, in *out).
+// grain: ranks per item, 0 = chosen problem by problem.
 // cfg (may be NULL) gives the shape of each FFT-size class it names; other
 // classes take ntm = 1, ipc = 1.
 int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, char *base,
@@ -47,7 +48,5 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
 // Clear accumulators, transpose factors, run the class kernels on
 // ctx->stream; the descriptor image must already be at `base`.
 int batch_issue(fcs_ctx *ctx, char *base, const BatchBuild &b);
-// About four work items per SM.
-int batch_default_grain(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q);
 
 }  // namespace fcs

@@ -15,6 +15,7 @@ struct BatchProb {
   int N, D, L, sb;
   int64_t R, rpi;
   int64_t I[kMaxN], off[kMaxN], ut_off[kMaxN];
+  int J[kMaxN];
   int64_t ldh, Jt;
   const float *UT;
   const int32_t *h;
@@ -26,7 +27,7 @@ struct BatchProb {
   int pad_;
 };
 
-// cp_run / cp13_run's accessors over a problem descriptor (fcs_cp_run.cuh).
+// cp_run / cp_pair_run's accessors over a problem descriptor (fcs_cp_run.cuh).
 struct BatchView {
   const BatchProb &P;
   int sb;
@@ -40,6 +41,11 @@ struct BatchView {
   __device__ __forceinline__ const float *column(int n, int64_t r) const {
     return P.UT + P.ut_off[n] + r * P.I[n];
   }
+  __device__ __forceinline__ float value(const float *col, int64_t i, int, int64_t) const {
+    return ld(col + i);
+  }
+  __device__ __forceinline__ int range(int n) const { return P.J[n]; }
+  __device__ __forceinline__ void ready() const {}
   __device__ __forceinline__ const int32_t *hashes(int d, int n) const {
     return P.h + d * P.ldh + P.off[n];
   }
@@ -57,6 +63,7 @@ struct ClassKernel {
   const void *fn;
   int nt;
   size_t smem;
+  int per_sm = 0;            // blocks that share an SM; 0 = as the runtime's occupancy says
 };
 
 // Threads of the slot FFT for log2 M = L at thread multiplier ntm (1: one
@@ -70,7 +77,7 @@ ClassKernel class_kernel_small(int L, int ntm, int ipc, int64_t Imax, int sb);  
 ClassKernel class_kernel_small2(int L, int ntm, int ipc, int64_t Imax, int sb); // L = 7 .. 9
 ClassKernel class_kernel_mid(int L, int ntm, int ipc, int64_t Imax, int sb);    // L = 10, 11
 ClassKernel class_kernel_12(int eng, int ntm, int ipc, int64_t Imax, int sb);   // L = 12
-ClassKernel class_kernel_13(int ipc, int64_t Imax, int sb);                     // L = 13
+ClassKernel class_kernel_13(int L, int ipc, int sb);                            // L = 13, 14
 
 // The kernels have internal linkage: each translation unit instantiates only
 // its own range of FFT sizes.
@@ -124,13 +131,17 @@ __global__ void __launch_bounds__(NT) batch_class_kernel(const BatchProb *__rest
   pdl_wait_previous();
 }
 
-// The same for P = 16384 on the warp-DIT engine (ra <= 32 RMAX).
-template <int CPT, int RMAX, bool MULTI>
-__global__ void __launch_bounds__(wdit::kNT) batch_class13_kernel(
-    const BatchProb *__restrict__ probs, const int4 *__restrict__ items,
-    const float2 *__restrict__ tw, int count, int ipc) {
+// The same for P = 1024 NR on the row-pair engine of fcs_pair.cuh.  The next
+// class may start once every CTA of this grid holds its tensor memory, so no
+// later class can hold what this one still waits for.
+template <int NR, bool MULTI>
+__global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
+    batch_pair_kernel(const BatchProb *__restrict__ probs, const int4 *__restrict__ items,
+                      const float2 *__restrict__ tw, int count, int ipc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int is_last;
+  __shared__ uint32_t slot;
+  const uint32_t tm = pfft::tmem_alloc<NR>(&slot);
   pdl_launch_dependents();
   auto one = [&](int it) {
     const int4 w = items[it];
@@ -138,7 +149,8 @@ __global__ void __launch_bounds__(wdit::kNT) batch_class13_kernel(
     const int64_t r0 = int64_t(w.z) * P.rpi;
     const int64_t r1 = min(P.R, r0 + P.rpi);
     const BatchView view{P, P.sb};
-    cp13_run<CPT, RMAX>(view, w.y, r0, r1, unsigned(P.groups), smem_raw, tw, &is_last);
+    cp_pair_run<NR, NR == 32 ? 8 : 4>(view, w.y, RankRange{r0, r1}, unsigned(P.groups), smem_raw,
+                                      tw, &is_last, tm);
   };
   if constexpr (MULTI) {
     const int first = blockIdx.x * ipc, last = min(count, first + ipc);
@@ -149,36 +161,16 @@ __global__ void __launch_bounds__(wdit::kNT) batch_class13_kernel(
   } else {
     one(blockIdx.x);
   }
+  pfft::tmem_free<NR>(tm);
   pdl_wait_previous();
 }
 
-// The same for P = 8192 on the warp-DIT engine of wdit::w12 (256 threads,
-// two CTAs per SM; ra <= 32 RMAX).
-template <int CPT, int RMAX, bool MULTI>
-__global__ void __launch_bounds__(wdit::w12::kNT, 2) batch_class12w_kernel(
-    const BatchProb *__restrict__ probs, const int4 *__restrict__ items,
-    const float2 *__restrict__ tw, int count, int ipc) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int is_last;
-  pdl_launch_dependents();
-  auto one = [&](int it) {
-    const int4 w = items[it];
-    const BatchProb &P = probs[w.x];
-    const int64_t r0 = int64_t(w.z) * P.rpi;
-    const int64_t r1 = min(P.R, r0 + P.rpi);
-    const BatchView view{P, P.sb};
-    cp12_run<CPT, RMAX>(view, w.y, r0, r1, unsigned(P.groups), smem_raw, tw, &is_last);
-  };
-  if constexpr (MULTI) {
-    const int first = blockIdx.x * ipc, last = min(count, first + ipc);
-    for (int it = first; it < last; ++it) {
-      if (it > first) __syncthreads();
-      one(it);
-    }
-  } else {
-    one(blockIdx.x);
-  }
-  pdl_wait_previous();
+template <int NR>
+ClassKernel pair_class_kernel(int ipc, int sb) {
+  const void *fn = ipc > 1 ? reinterpret_cast<const void *>(batch_pair_kernel<NR, true>)
+                           : reinterpret_cast<const void *>(batch_pair_kernel<NR, false>);
+  const size_t smem = pfft::Smem<NR>::bytes((sb + 2 * NR - 1) / (2 * NR));
+  return ClassKernel{fn, pfft::Geo<NR>::NT, smem, pfft::blocks_per_sm<NR>(smem)};
 }
 
 // Slot-FFT class kernel for log2 M = L with NT threads: prefetch depth from

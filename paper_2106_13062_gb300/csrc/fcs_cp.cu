@@ -36,9 +36,14 @@ struct CpArgs {
   const int32_t *h;
   const int8_t *s;
   float2 *G;             // [D][M+2] spectrum accumulator (bins 0..M), zeroed per call
-  unsigned *counter;     // [D] tickets, zero at launch, reset by the last CTA
+  unsigned *counter;     // [kMaxD] tickets, zero at launch, reset by the last CTA; then [kMaxD]
+                         // 64-bit rank counters of the row-pair engine, zero at launch
   float *out;            // [D][Jt]
   int sb;                // scatter buffer length (floats): max J_n rounded up to 4
+  // CpStridedView only: the factor matrices in place
+  const float *U[kMaxN];
+  int64_t ldU[kMaxN];
+  const float *lambda;
 };
 
 // All modes in one launch: mode n = blockIdx.z.
@@ -50,7 +55,18 @@ struct TransposeArgs {
   float *UT;
 };
 
-// cp_run / cp13_run's accessors over CpArgs (fcs_cp_run.cuh).
+// The sketch kernels of fcs_sketch_cp are launched as programmatic dependents
+// of the prep launch, so their CTAs are placed while prep runs.  Every one of
+// them waits for the prep grid to complete (and its writes to be visible:
+// transposed factors, cleared accumulator and tickets, hash tables) before
+// anything that touches those: cp_kernel first of all, cp_pair_kernel once
+// its tables and scatter buffer are set up.  Launched the ordinary way the
+// wait returns at once.
+__device__ __forceinline__ void wait_for_prep() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// cp_run / cp_pair_run's accessors over CpArgs (fcs_cp_run.cuh).
 struct CpView {
   const CpArgs &a;
   int sb;
@@ -67,6 +83,11 @@ struct CpView {
   __device__ __forceinline__ const float *column(int n, int64_t r) const {
     return a.UT + a.ut_off[n] + r * a.m.I[n];
   }
+  __device__ __forceinline__ float value(const float *col, int64_t i, int, int64_t) const {
+    return ld(col + i);
+  }
+  __device__ __forceinline__ int range(int n) const { return a.m.J[n]; }
+  __device__ __forceinline__ void ready() const { wait_for_prep(); }
   __device__ __forceinline__ const int32_t *hashes(int d, int n) const {
     return a.h + d * a.m.ldh + a.m.off[n];
   }
@@ -79,14 +100,27 @@ struct CpView {
   __device__ __forceinline__ unsigned *ticket(int d) const { return a.counter + d; }
 };
 
-// The sketch kernels of fcs_sketch_cp are launched as programmatic dependents
-// of the prep launch, so their CTAs are placed while prep runs.  Every one of
-// them waits for the prep grid to complete (and its writes to be visible:
-// transposed factors, cleared accumulator and tickets, hash tables) before
-// anything else; launched the ordinary way the wait returns at once.
-__device__ __forceinline__ void wait_for_prep() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+// The same with the factor columns read in place (row stride ldU), for a
+// caller without room for the transposed copy.
+struct CpStridedView : CpView {
+  __device__ __forceinline__ const float *column(int n, int64_t r) const { return a.U[n] + r; }
+  __device__ __forceinline__ float value(const float *col, int64_t i, int n, int64_t r) const {
+    const float v = __ldg(col + i * a.ldU[n]);
+    return n == 0 && a.lambda ? v * __ldg(a.lambda + r) : v;
+  }
+};
+
+template <class View>
+__device__ __forceinline__ View make_view(const CpArgs &a) {
+  if constexpr (std::is_same<View, CpView>::value)
+    return CpView{a, a.sb};
+  else
+    return View{CpView{a, a.sb}};
 }
+
+// Factor entries fetched ahead per thread on the row-pair engine (the rest of
+// a longer column is loaded when it is scattered).
+constexpr int pair_cpt(int NR) { return NR == 32 ? 8 : 4; }
 
 // CTA (g, d): ranks [g * ranks_per_cta, ...) of sketch d.
 template <int LOG2M, int NT, int CPT>
@@ -100,31 +134,25 @@ __global__ void __launch_bounds__(NT) cp_kernel(CpArgs a, const float2 *__restri
   cp_run<LOG2M, NT, CPT>(view, blockIdx.y, r0, r1, gridDim.x, smem_raw, tw, &is_last);
 }
 
-// The same for P = 16384 on the warp-DIT engine.  RMAX = number of 32-entry
-// blocks per scatter-buffer row (ra <= 32 RMAX).
-template <int CPT, int RMAX>
-__global__ void __launch_bounds__(wdit::kNT) cp13_kernel(CpArgs a, const float2 *__restrict__ tw) {
-  wait_for_prep();
+// The same for P = 1024 NR on the row-pair engine.  A one-dimensional grid:
+// block b works on sketch b mod D, whose blocks share its ranks through a
+// counter (a fixed split left the SMs idle a fifth of the time: the blocks of
+// three and of four ranks do not pair up evenly on the SMs).
+template <int NR, class View>
+__global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
+    cp_pair_kernel(CpArgs a, const float2 *__restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int is_last;
-  const int64_t r0 = blockIdx.x * a.ranks_per_cta;
-  const int64_t r1 = min(a.R, r0 + a.ranks_per_cta);
-  const CpView view{a, a.sb};
-  cp13_run<CPT, RMAX>(view, blockIdx.y, r0, r1, gridDim.x, smem_raw, tw, &is_last);
-}
-
-// The same for P = 8192 on the warp-DIT engine (256 threads, two CTAs per
-// SM).  RMAX = number of 32-entry blocks per scatter-buffer row.
-template <int CPT, int RMAX>
-__global__ void __launch_bounds__(wdit::w12::kNT, 2) cp12_kernel(CpArgs a,
-                                                                 const float2 *__restrict__ tw) {
-  wait_for_prep();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int is_last;
-  const int64_t r0 = blockIdx.x * a.ranks_per_cta;
-  const int64_t r1 = min(a.R, r0 + a.ranks_per_cta);
-  const CpView view{a, a.sb};
-  cp12_run<CPT, RMAX>(view, blockIdx.y, r0, r1, gridDim.x, smem_raw, tw, &is_last);
+  __shared__ uint32_t slot;
+  __shared__ int64_t next_rank;
+  const uint32_t tm = pfft::tmem_alloc<NR>(&slot);
+  const unsigned groups = gridDim.x / unsigned(a.D);
+  const int g = int(blockIdx.x) / a.D, d = int(blockIdx.x) - g * a.D;
+  const View view = make_view<View>(a);
+  const RankQueue ranks{a.R, groups, unsigned(g),
+                        reinterpret_cast<unsigned long long *>(a.counter + kMaxD) + d, &next_rank};
+  cp_pair_run<NR, pair_cpt(NR)>(view, d, ranks, groups, smem_raw, tw, &is_last, tm);
+  pfft::tmem_free<NR>(tm);
 }
 
 // prep_kernel: in one launch, the factor transpose in 32 x 32 tiles,
@@ -187,30 +215,15 @@ __global__ void __launch_bounds__(256) prep_kernel(PrepArgs a) {
   if (e < a.hs.total) hash_entry(a.hs, d, e, a.h, a.s);
 }
 
-// Kernel for the given prefetch depth and scatter-buffer height.
-template <int CPT>
-const void *cp13_pick_rmax(int ra) {
-  if (ra <= 128) return reinterpret_cast<const void *>(cp13_kernel<CPT, 4>);
-  if (ra <= 256) return reinterpret_cast<const void *>(cp13_kernel<CPT, 8>);
-  return reinterpret_cast<const void *>(cp13_kernel<CPT, 16>);
-}
-const void *cp13_pick(int64_t Imax, int sb) {
-  const int ra = (sb + 31) >> 5;
-  const int cpt = int((Imax + wdit::kNT - 1) / wdit::kNT);
-  if (cpt <= 1) return cp13_pick_rmax<1>(ra);
-  if (cpt <= 2) return cp13_pick_rmax<2>(ra);
-  return cp13_pick_rmax<4>(ra);
-}
-
 // Launch a sketch kernel as a programmatic dependent of the prep launch
 // before it on the context's stream.
-cudaError_t launch_after_prep(fcs_ctx *ctx, const void *kern, dim3 grid, dim3 block, size_t smem,
-                              void **args) {
+cudaError_t launch_after_prep(cudaStream_t st, const void *kern, dim3 grid, dim3 block,
+                              size_t smem, void **args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = ctx->stream;
+  cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -219,62 +232,46 @@ cudaError_t launch_after_prep(fcs_ctx *ctx, const void *kern, dim3 grid, dim3 bl
   return cudaLaunchKernelExC(&cfg, kern, args);
 }
 
-int launch_cp13(fcs_ctx *ctx, CpArgs &a, int64_t groups, int64_t Imax) {
-  const size_t smem = Cp13Smem::bytes((a.sb + 31) >> 5);
-  const void *kern = cp13_pick(Imax, a.sb);
-  cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(cp13)");
-  const float2 *twp = ctx->twiddle;
-  void *args[] = {&a, &twp};
-  e = launch_after_prep(ctx, kern, dim3(unsigned(groups), unsigned(a.D)), dim3(wdit::kNT), smem,
-                        args);
-  return check_cuda(ctx, e, "cp13_kernel");
+// Rank groups per sketch on the row-pair engine: the CTAs that the GPU holds
+// at once, spread over the sketches.
+template <int NR>
+int64_t pair_groups(int sm_count, int64_t R, int D, size_t smem) {
+  const int per_sm = pfft::blocks_per_sm<NR>(smem);
+  return std::max<int64_t>(1, std::min<int64_t>(R, int64_t(sm_count) * per_sm / D));
 }
 
-template <int CPT>
-const void *cp12_pick_rmax(int ra) {
-  if (ra <= 128) return reinterpret_cast<const void *>(cp12_kernel<CPT, 4>);
-  if (ra <= 256) return reinterpret_cast<const void *>(cp12_kernel<CPT, 8>);
-  return reinterpret_cast<const void *>(cp12_kernel<CPT, 16>);
-}
-
-int launch_cp12(fcs_ctx *ctx, CpArgs &a, int64_t groups, int64_t Imax) {
-  const int ra = (a.sb + 15) >> 4;
-  const size_t smem = Cp12Smem::bytes(ra);
-  const int cpt = int((Imax + wdit::w12::kNT - 1) / wdit::w12::kNT);
-  const void *kern = cpt <= 1 ? cp12_pick_rmax<1>(ra) : cpt <= 2 ? cp12_pick_rmax<2>(ra)
-                                                                 : cp12_pick_rmax<4>(ra);
-  cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(cp12)");
-  const float2 *twp = ctx->twiddle;
-  void *args[] = {&a, &twp};
-  e = launch_after_prep(ctx, kern, dim3(unsigned(groups), unsigned(a.D)), dim3(wdit::w12::kNT),
-                        smem, args);
-  return check_cuda(ctx, e, "cp12_kernel");
+// Row-pair kernel launch on `st` (a programmatic dependent of the prep launch
+// before it).
+template <int NR, class View>
+cudaError_t launch_pair(CpArgs &a, int sm_count, const float2 *tw, cudaStream_t st) {
+  const size_t smem = pfft::Smem<NR>::bytes((a.sb + 2 * NR - 1) / (2 * NR));
+  const void *kern = reinterpret_cast<const void *>(cp_pair_kernel<NR, View>);
+  const cudaError_t e = allow_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t groups = pair_groups<NR>(sm_count, a.R, a.D, smem);
+  void *args[] = {&a, &tw};
+  return launch_after_prep(st, kern, dim3(unsigned(groups * a.D)), dim3(pfft::Geo<NR>::NT), smem,
+                           args);
 }
 
 template <int LOG2M>
 int launch_cp(fcs_ctx *ctx, CpArgs &a, int64_t groups, int64_t Imax) {
-  if constexpr (LOG2M == wdit::kL) {
-    return launch_cp13(ctx, a, groups, Imax);
-  } else if constexpr (LOG2M == 12) {
-    return launch_cp12(ctx, a, groups, Imax);
+  if constexpr (LOG2M >= 12) {
+    return check_cuda(ctx,
+                      launch_pair<1 << (LOG2M - 9), CpView>(a, ctx->sm_count, ctx->twiddle,
+                                                            ctx->stream),
+                      "cp_pair_kernel");
   } else {
     constexpr int NT = fft_threads(LOG2M);
     const size_t smem = CpSmem<LOG2M, NT>::bytes(a.sb);
     const int cpt = int((Imax + NT - 1) / NT);
     auto go = [&](auto kern) -> int {
-      if (smem > 48 * 1024) {
-        cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(cp)");
-      }
+      const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), smem);
+      if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(cp)");
       const float2 *twp = ctx->twiddle;
       void *args[] = {&a, &twp};
       return check_cuda(ctx,
-                        launch_after_prep(ctx, reinterpret_cast<const void *>(kern),
+                        launch_after_prep(ctx->stream, reinterpret_cast<const void *>(kern),
                                           dim3(unsigned(groups), unsigned(a.D)), dim3(NT), smem,
                                           args),
                         "cp_kernel");
@@ -323,7 +320,24 @@ int sketch_cp_impl(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t *ho
   if (log2p > kMaxLog2PBig)
     return set_error(ctx, FCS_EUNSUPPORTED, "Jt=%lld needs FFT length > %d",
                      (long long)a.m.Jt, 1 << kMaxLog2PBig);
-  if (log2p > kMaxLog2P) {
+  const int log2m = log2p - 1;
+  const int M = 1 << log2m;
+  int64_t Imax = 0, Jmax = 0, utlen = 0;
+  for (int n = 0; n < N; ++n) {
+    a.ut_off[n] = utlen;
+    utlen += R * host_I[n];
+    if (host_I[n] > Imax) Imax = host_I[n];
+    if (host_J[n] > Jmax) Jmax = host_J[n];
+  }
+  const size_t gbytes = (sizeof(float2) * size_t(D) * size_t(M + 2) + 255) & ~size_t(255);
+  const size_t cbytes = 256;
+  const size_t wbytes = gbytes + cbytes + sizeof(float) * size_t(utlen);
+  // P = 32768 runs here too when its scatter buffer fits shared memory and
+  // the transposed factors fit the workspace of a long call
+  const bool here = log2p <= kMaxLog2P ||
+                    (log2p == kMaxLog2P + 1 && Jmax <= kPair32MaxJ &&
+                     ((wbytes + 255) & ~size_t(255)) <= std::min(ctx->budget, size_t(512) << 20));
+  if (!here) {
     if (gen) {                          // long route: tables by their own launch
       rc = fcs_make_hashes(ctx, gen->seed, N, host_I, host_J, D, gen->h, gen->s);
       if (rc) return rc;
@@ -332,34 +346,21 @@ int sketch_cp_impl(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t *ho
     spec_cache_invalidate(ctx, out, sizeof(float) * size_t(D) * size_t(a.m.Jt));
     return big_sketch_cp(ctx, a.m, R, D, host_U, host_ldU, lambda, h, s, out, log2p);
   }
-  const int log2m = log2p - 1;
-  const int M = 1 << log2m;
   a.D = D;
   a.R = R;
   a.h = h;
   a.s = s;
   a.out = out;
-  // rank groups: about one CTA per SM over all sketches (two for P = 8192,
-  // whose engine fits two CTAs per SM)
-  const int64_t slots = int64_t(ctx->sm_count) * (log2m == 12 ? 2 : 1);
-  int64_t groups = (slots + D - 1) / D;
+  // rank groups of the slot FFT: about one CTA per SM over all sketches
+  int64_t groups = (int64_t(ctx->sm_count) + D - 1) / D;
   if (groups < 1) groups = 1;
   if (groups > R) groups = R;
   a.ranks_per_cta = (R + groups - 1) / groups;
   groups = (R + a.ranks_per_cta - 1) / a.ranks_per_cta;
 
-  int64_t Imax = 0, Jmax = 0, utlen = 0;
-  for (int n = 0; n < N; ++n) {
-    a.ut_off[n] = utlen;
-    utlen += R * host_I[n];
-    if (host_I[n] > Imax) Imax = host_I[n];
-    if (host_J[n] > Jmax) Jmax = host_J[n];
-  }
   a.sb = int((Jmax + 3) / 4 * 4);
-  const size_t gbytes = (sizeof(float2) * size_t(D) * size_t(M + 2) + 255) & ~size_t(255);
-  const size_t cbytes = 256;
   void *ws = nullptr;
-  rc = ensure_workspace(ctx, gbytes + cbytes + sizeof(float) * size_t(utlen), &ws);
+  rc = ensure_workspace(ctx, wbytes, &ws);
   if (rc) return rc;
   a.G = static_cast<float2 *>(ws);
   a.counter = reinterpret_cast<unsigned *>(static_cast<char *>(ws) + gbytes);
@@ -399,12 +400,49 @@ int sketch_cp_impl(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t *ho
     rc = check_cuda(ctx, cudaGetLastError(), "prep_kernel");
     if (rc) return rc;
   }
+  if (log2m == 14)
+    return check_cuda(ctx, launch_pair<32, CpView>(a, ctx->sm_count, ctx->twiddle, ctx->stream),
+                      "cp_pair_kernel");
   rc = FCS_EUNSUPPORTED;
   FCS_DISPATCH_LOG2M(log2m, rc = launch_cp<L>(ctx, a, groups, Imax));
   return rc;
 }
 
 }  // namespace
+
+// The P = 32768 sketch with the factors read in place (Jmax <= kPair32MaxJ),
+// for callers whose memory does not hold their transposed copy: `ws` has
+// pair32_strided_bytes(D).
+size_t fcs::pair32_strided_bytes(int D) {
+  return ((sizeof(float2) * size_t(D) * size_t((1 << 14) + 2) + 255) & ~size_t(255)) + 256;
+}
+int fcs::pair32_sketch_strided(fcs_ctx *ctx, const Modes &m, int64_t R, int D,
+                               const float *const *host_U, const int64_t *host_ldU,
+                               const float *lambda, const int32_t *h, const int8_t *s, float *out,
+                               void *ws) {
+  CpArgs a{};
+  a.m = m;
+  a.D = D;
+  a.R = R;
+  a.h = h;
+  a.s = s;
+  a.out = out;
+  int Jmax = 1;
+  for (int n = 0; n < m.N; ++n) {
+    a.U[n] = host_U[n];
+    a.ldU[n] = host_ldU[n];
+    Jmax = std::max(Jmax, int(m.J[n]));
+  }
+  a.lambda = lambda;
+  a.sb = (Jmax + 3) / 4 * 4;
+  const size_t bytes = pair32_strided_bytes(D);
+  a.G = static_cast<float2 *>(ws);
+  a.counter = reinterpret_cast<unsigned *>(static_cast<char *>(ws) + bytes - 256);
+  int rc = check_cuda(ctx, cudaMemsetAsync(ws, 0, bytes, ctx->stream), "cudaMemsetAsync(G)");
+  if (rc) return rc;
+  return check_cuda(ctx, launch_pair<32, CpStridedView>(a, ctx->sm_count, ctx->twiddle, ctx->stream),
+                    "cp_pair_kernel");
+}
 
 extern "C" int fcs_sketch_cp(fcs_ctx *ctx, int N, const int64_t *host_I,
                              const int32_t *host_J, int64_t R, int D,
@@ -506,37 +544,30 @@ int noalloc_setup(int dev, cudaStream_t st, NoAllocDevice **out, char *err, size
 }
 
 template <int LOG2M>
-int noalloc_launch_cp(CpArgs &a, int64_t groups, int64_t Imax, const float2 *tw,
+int noalloc_launch_cp(CpArgs &a, int64_t groups, int64_t Imax, int sm_count, const float2 *tw,
                       cudaStream_t st, char *err, size_t n) {
-  constexpr int NT = fft_threads(LOG2M);
-  const size_t smem = LOG2M == wdit::kL ? Cp13Smem::bytes((a.sb + 31) >> 5)
-                                        : CpSmem<LOG2M, NT>::bytes(a.sb);
-  const int cpt = int((Imax + NT - 1) / NT);
-  auto go = [&](auto kern) -> int {
-    if (smem > 48 * 1024) {
-      cudaError_t e =
-          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-      if (e != cudaSuccess)
-        return noalloc_fail(err, n, FCS_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
-    kern<<<dim3(unsigned(groups), unsigned(a.D)), NT, smem, st>>>(a, tw);
-    cudaError_t e = cudaGetLastError();
+  if constexpr (LOG2M >= 12) {
+    const cudaError_t e = launch_pair<1 << (LOG2M - 9), CpView>(a, sm_count, tw, st);
     if (e != cudaSuccess)
-      return noalloc_fail(err, n, FCS_ECUDA, "cp_kernel: %s", cudaGetErrorString(e));
-    return FCS_OK;
-  };
-  if constexpr (LOG2M == wdit::kL) {
-    const void *kern = cp13_pick(Imax, a.sb);
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess)
-      return noalloc_fail(err, n, FCS_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    void *args[] = {&a, &tw};
-    e = cudaLaunchKernel(kern, dim3(unsigned(groups), unsigned(a.D)), dim3(NT), args, smem, st);
-    if (e != cudaSuccess)
-      return noalloc_fail(err, n, FCS_ECUDA, "cp13_kernel: %s", cudaGetErrorString(e));
+      return noalloc_fail(err, n, FCS_ECUDA, "cp_pair_kernel: %s", cudaGetErrorString(e));
     return FCS_OK;
   } else {
+    constexpr int NT = fft_threads(LOG2M);
+    const size_t smem = CpSmem<LOG2M, NT>::bytes(a.sb);
+    const int cpt = int((Imax + NT - 1) / NT);
+    auto go = [&](auto kern) -> int {
+      {
+        const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), smem);
+        if (e != cudaSuccess)
+          return noalloc_fail(err, n, FCS_ECUDA, "cudaFuncSetAttribute: %s",
+                              cudaGetErrorString(e));
+      }
+      kern<<<dim3(unsigned(groups), unsigned(a.D)), NT, smem, st>>>(a, tw);
+      cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess)
+        return noalloc_fail(err, n, FCS_ECUDA, "cp_kernel: %s", cudaGetErrorString(e));
+      return FCS_OK;
+    };
     if (cpt <= 1) return go(cp_kernel<LOG2M, NT, 1>);
     if (cpt <= 2) return go(cp_kernel<LOG2M, NT, 2>);
     return go(cp_kernel<LOG2M, NT, 4>);
@@ -641,7 +672,7 @@ extern "C" int fcs_sketch_cp_noalloc(void *stream, int N, const int64_t *host_I,
       return noalloc_fail(err, err_len, FCS_ECUDA, "prep: %s", cudaGetErrorString(e));
   }
   rc = FCS_EUNSUPPORTED;
-  FCS_DISPATCH_LOG2M(log2m, rc = noalloc_launch_cp<L>(a, groups, Imax, sd->twiddle, st, err,
-                                                      err_len));
+  FCS_DISPATCH_LOG2M(log2m, rc = noalloc_launch_cp<L>(a, groups, Imax, sd->sm_count, sd->twiddle, st,
+                                                      err, err_len));
   return rc;
 }

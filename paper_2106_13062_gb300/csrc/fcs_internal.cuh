@@ -88,6 +88,17 @@ struct DeviceGuard {
   }
 };
 
+// Let a kernel be launched with up to `bytes` of dynamic shared memory.  The
+// limit is always set to the same value, beyond which no kernel here goes: it
+// belongs to the kernel and not to a launch, so a smaller value set for one
+// launch would refuse another, larger one that was prepared before it.
+constexpr size_t kMaxDynSmem = 232448 - 1024;      // 227 KiB less room for static arrays
+inline cudaError_t allow_smem(const void *kern, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              int(bytes > kMaxDynSmem ? bytes : kMaxDynSmem));
+}
+
 inline int ilog2_ceil(int64_t x) {
   int l = 0;
   while ((int64_t(1) << l) < x) ++l;
@@ -175,21 +186,27 @@ __device__ __forceinline__ void bfly_tw(float2 &a, float2 &b) {
   b = make_float2(fmaf(-f, ux, a0.x), fmaf(-f, uy, a0.y));
 }
 
+// x = a - i b, y = a + i b.
+__device__ __forceinline__ void bfly_mi(float2 a, float2 b, float2 &x, float2 &y) {
+  x = make_float2(a.x + b.y, a.y - b.x);
+  y = make_float2(a.x - b.y, a.y + b.x);
+}
+
 // Last radix-2 stage of an R-point DFT from the half-size DFTs e (even
 // inputs) and o (odd inputs): v[k] = e[k] + W_R^k o[k], v[k + R/2] =
 // e[k] - W_R^k o[k], unrolled over k by template recursion.
+// (E: the element type, float2 or a pair of complex numbers.)
 template <int R, int K = 0>
 struct DftCombine {
-  static __device__ __forceinline__ void run(float2 *v, const float2 *e, const float2 *o) {
+  template <class E>
+  static __device__ __forceinline__ void run(E *v, const E *e, const E *o) {
     if constexpr (K < R / 2) {
-      float2 a = e[K], b = o[K];
+      E a = e[K], b = o[K];
       if constexpr (K == 0) {
         v[K] = cadd(a, b);
         v[K + R / 2] = csub(a, b);
       } else if constexpr (4 * K == R) {                 // W = -i
-        const float2 t = make_float2(b.y, -b.x);
-        v[K] = cadd(a, t);
-        v[K + R / 2] = csub(a, t);
+        bfly_mi(a, b, v[K], v[K + R / 2]);
       } else {
         bfly_tw<K * (64 / R)>(a, b);
         v[K] = a;
@@ -204,8 +221,9 @@ struct DftCombine {
 // order in and out: X[k] = sum_n x[n] exp(-2 pi i n k / R).
 template <int R>
 struct Dft {
-  static __device__ __forceinline__ void run(float2 *v) {
-    float2 e[R / 2], o[R / 2];
+  template <class E>
+  static __device__ __forceinline__ void run(E *v) {
+    E e[R / 2], o[R / 2];
 #pragma unroll
     for (int k = 0; k < R / 2; ++k) {
       e[k] = v[2 * k];
@@ -218,7 +236,36 @@ struct Dft {
 };
 template <>
 struct Dft<1> {
-  static __device__ __forceinline__ void run(float2 *) {}
+  template <class E>
+  static __device__ __forceinline__ void run(E *) {}
+};
+
+// DFT of size R whose inputs v[NZ..R-1] are zero (input-pruned radix-2
+// decimation in time; entries at or past NZ are not read).
+template <int R, int NZ>
+struct DftNZ {
+  template <class E>
+  static __device__ __forceinline__ void run(E *v) {
+    if constexpr (NZ >= R) {
+      Dft<R>::run(v);
+    } else if constexpr (NZ <= 0) {
+#pragma unroll
+      for (int k = 0; k < R; ++k) v[k] = E{};
+    } else if constexpr (NZ == 1) {
+#pragma unroll
+      for (int k = 1; k < R; ++k) v[k] = v[0];
+    } else {
+      E e[R / 2], o[R / 2];
+#pragma unroll
+      for (int k = 0; k < R / 2; ++k) {
+        e[k] = v[2 * k];
+        o[k] = v[2 * k + 1];
+      }
+      DftNZ<R / 2, (NZ + 1) / 2>::run(e);
+      DftNZ<R / 2, NZ / 2>::run(o);
+      DftCombine<R>::run(v, e, o);
+    }
+  }
 };
 
 // One Stockham auto-sort pass of radix R over a length-M sequence in padded
@@ -503,17 +550,21 @@ int make_modes_msg(char *err, size_t n, int N, const int64_t *host_I,
 // FFT-based calls for kMaxLog2P < log2p <= kMaxLog2PBig (fcs_big.cu); the
 // callers have validated the arguments.
 // ext_ws: caller-owned device buffer of ext_bytes (a batch plan's), or NULL
-// for the context workspace.  stage 0 issues everything.  A batch plan splits
-// the P = 2^15 warp-DIT route in two: stage 1 issues only the clearing of its
-// accumulator (*split = true when the route applies; otherwise nothing is
-// issued), stage 2 only its kernel, launched as a programmatic dependent of
-// the kernel before it in the stream (it waits for that grid at its end).
+// for the context workspace.
 int big_sketch_cp(fcs_ctx *ctx, const Modes &m, int64_t R, int D, const float *const *host_U,
                   const int64_t *host_ldU, const float *lambda, const int32_t *h,
                   const int8_t *s, float *out, int log2p, void *ext_ws = nullptr,
-                  size_t ext_bytes = 0, int stage = 0, bool *split = nullptr);
+                  size_t ext_bytes = 0);
 // Device bytes big_sketch_cp uses when its buffer holds at most `cap` bytes.
 size_t big_sketch_cp_bytes(const Modes &m, int64_t R, int D, int log2p, size_t cap, int nsm);
+// The longest hash range of a P = 32768 CP sketch whose scatter buffer fits
+// shared memory on the row-pair engine (fcs_pair.cuh).
+constexpr int kPair32MaxJ = 17984;
+size_t pair32_strided_bytes(int D);
+int pair32_sketch_strided(fcs_ctx *ctx, const Modes &m, int64_t R, int D,
+                          const float *const *host_U, const int64_t *host_ldU,
+                          const float *lambda, const int32_t *h, const int8_t *s, float *out,
+                          void *ws);
 int big_contract(fcs_ctx *ctx, const Modes &m, int kind, int free_mode, int D,
                  const float *fcsT, int64_t B, const float *const *vec, const int32_t *h,
                  const int8_t *s, float2 *spec, bool need_spec, cudaEvent_t spec_ready,

@@ -407,7 +407,7 @@ int issue_round(fcs_server *S, int si, std::vector<Req *> &reqs, Round &rd) {
   }
   // one batched launch for every CP request of the round
   if (!probs.empty()) {
-    const int grain = fcs::batch_default_grain(ctx, int(probs.size()), probs.data());
+    const int grain = 0;
     fcs::BatchBuild bb{};
     std::vector<char> desc;
     int rc = fcs::batch_build(ctx, int(probs.size()), probs.data(), grain, nullptr, &desc, &bb);
