@@ -8,7 +8,7 @@
 // Fast path (last mode contiguous, 16-byte aligned rows): one warp handles
 // 128 consecutive entries of a row with one float4 load per lane; the partial
 // hash of the leading modes is computed once per row and sketch.
-#include "fcs_internal.cuh"
+#include "fcs_dense_items.cuh"
 
 #include <cfloat>
 #include <type_traits>
@@ -661,6 +661,12 @@ extern "C" int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
 
   DeviceGuard g(ctx->device);
   spec_cache_invalidate(ctx, out, sizeof(float) * size_t((nbatch - 1) * a.obs + D * Jt));
+  {
+    bool done = false;
+    rc = dense_items(ctx, N, a.m.I, a.stride, a.m.off, a.m.J, a.m.ldh, Jt, D, T, h, s, out, nbatch,
+                     a.tbs, a.obs, &done);
+    if (rc || done) return rc;
+  }
   // zero the output sketches
   {
     int64_t len = D * Jt;

@@ -6,12 +6,15 @@
 // i.e. per sketch d the product of the [B][Jt] activation sketches with the
 // transposed [C][Jt] weight sketches, then the median over the D sketches.
 //
-// The product kernel tiles (b, c) by 64 x 64 per CTA (256 threads, 4 x 4
+// Two kernels.  inner_kernel tiles (b, c) by 64 x 64 per CTA (256 threads, 4 x 4
 // outputs each), stages 32-bin slices of both operands in shared memory and
 // accumulates in FP32 registers, one sketch d per grid z; the median kernel
-// then reads the D values of each output.  The sketch is Jt long and B, C
-// are batch and class counts, so this is a small dense contraction on the
-// FP32 pipe; it is not the hot path.
+// then reads the D values of each output.  When that grid would leave SMs
+// without a CTA (a layer's batch and class counts: 256 x 10 at D = 5 makes 20
+// CTAs, 36 us), inner_small_kernel gives every 4 x 4 outputs a CTA of D warps,
+// one sketch each with the lanes along the bins, and takes the medians itself:
+// 6 us there, and one launch less (Jt = 1000, D = 5: 1 x 10 outputs 8 us for 70,
+// 256 x 200 38 for 128; 512 x 1000, where the tiles fill the SMs, stays at 295).
 #include "fcs_internal.cuh"
 
 namespace fcs {
@@ -65,6 +68,65 @@ __global__ void __launch_bounds__(256) inner_kernel(const float *__restrict__ sa
     }
 }
 
+// Outputs (4 blockIdx.y + i, 4 blockIdx.x + q), i, q < 4; warp d sums sketch d.
+template <int D>
+__global__ void __launch_bounds__(32 * D) inner_small_kernel(
+    const float *__restrict__ sa, const float *__restrict__ sw, int64_t B, int64_t C, int64_t Jt,
+    const float *__restrict__ bias, float *__restrict__ out, float *__restrict__ raw) {
+  __shared__ float val[D][16];
+  const int d = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t b0 = 4 * int64_t(blockIdx.y), c0 = 4 * int64_t(blockIdx.x);
+  const float *pa[4], *pw[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {            // rows past the end repeat the last one
+    pa[i] = sa + (min(b0 + i, B - 1) * D + d) * Jt;
+    pw[i] = sw + (min(c0 + i, C - 1) * D + d) * Jt;
+  }
+  float acc[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+#pragma unroll 2
+  for (int64_t j = lane; j < Jt; j += 32) {
+    float a[4], w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a[i] = __ldg(pa[i] + j);
+      w[i] = __ldg(pw[i] + j);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[4 * i + q] = fmaf(a[i], w[q], acc[4 * i + q]);
+  }
+  // lane l ends with output l mod 16 summed over its half-warp, then both
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < o; ++k) {
+      const float give = up ? acc[k] : acc[k + o];
+      const float keep = up ? acc[k + o] : acc[k];
+      acc[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 16);
+  if (lane < 16) val[d][lane] = acc[0];
+  __syncthreads();
+  if (threadIdx.x < 16) {
+    const int64_t b = b0 + (threadIdx.x >> 2), c = c0 + (threadIdx.x & 3);
+    if (b < B && c < C) {
+      float v[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        v[k] = val[k][threadIdx.x];
+        if (raw) raw[(b * C + c) * D + k] = v[k];
+      }
+      const float m = median_net<D>(v);
+      out[b * C + c] = bias ? m + __ldg(bias + c) : m;
+    }
+  }
+}
+
 template <int D>
 __global__ void median_bias_kernel(const float *__restrict__ raw, int64_t BC, int64_t C,
                                    const float *__restrict__ bias, float *__restrict__ out) {
@@ -94,6 +156,23 @@ extern "C" int fcs_sketch_inner(fcs_ctx *ctx, int D, int64_t Jt, int64_t B, cons
     return set_error(ctx, FCS_EINVAL, "B=%lld too large", (long long)B);
   if (!sa || !sw || !out_median) return set_error(ctx, FCS_EINVAL, "NULL pointer argument");
   DeviceGuard g(ctx->device);
+  if (((B + kTile - 1) / kTile) * ((C + kTile - 1) / kTile) * D < ctx->sm_count) {
+    const dim3 gs(unsigned((C + 3) / 4), unsigned((B + 3) / 4));
+    switch (D) {
+#define FCS_IS_CASE(K)                                                                            \
+  case K:                                                                                         \
+    inner_small_kernel<K><<<gs, 32 * K, 0, ctx->stream>>>(sa, sw, B, C, Jt, bias, out_median,     \
+                                                          out_raw);                               \
+    break;
+      FCS_IS_CASE(1) FCS_IS_CASE(2) FCS_IS_CASE(3) FCS_IS_CASE(4) FCS_IS_CASE(5)
+      FCS_IS_CASE(6) FCS_IS_CASE(7) FCS_IS_CASE(8) FCS_IS_CASE(9) FCS_IS_CASE(10)
+      FCS_IS_CASE(11) FCS_IS_CASE(12) FCS_IS_CASE(13) FCS_IS_CASE(14) FCS_IS_CASE(15)
+      FCS_IS_CASE(16)
+#undef FCS_IS_CASE
+      default: break;
+    }
+    return check_cuda(ctx, cudaGetLastError(), "inner_small_kernel");
+  }
   float *raw = out_raw;
   if (!raw) {
     int rc = ensure_raw(ctx, sizeof(float) * size_t(B) * size_t(C) * D);

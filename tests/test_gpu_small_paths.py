@@ -1,0 +1,90 @@
+"""Kernels for small work against the FP64 oracle or FP64 numpy at the sizes
+where they can go wrong: dense sketches of small tensors (one block per
+tensor), inner products of few sketches, and the ALS update at every rank
+class.  Needs a GPU."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import synth
+from gpu_common import CONTRACT_RTOL, assert_sketch_close, cuda, host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fcs():
+    import paper_2106_13062_gb300 as m
+    m.build()
+    return m
+
+
+@pytest.fixture(scope="module")
+def ctx(fcs):
+    c = fcs.Context()
+    yield c
+    c.close()
+
+
+def _dense_ref(orc, T, J, ho, so):
+    return np.stack([orc.fcs_dense(t.astype(np.float64), J, ho, so) for t in T])
+
+
+@pytest.mark.parametrize("shape,J,D,nb", [
+    ((1,), [1], 1, 1), ((7, 7, 32), [60, 60, 60], 5, 400), ((3, 5, 7), [4, 9, 11], 3, 1),
+    ((2, 1, 3, 1, 2), [3, 2, 5, 1, 4], 16, 5), ((8192,), [300], 4, 200), ((91, 90), [50, 70], 2, 160),
+    ((8193,), [3000], 1, 160), ((33, 31), [16384, 16384], 1, 160), ((64, 64), [90, 80], 1, 3),
+])
+@pytest.mark.parametrize("kind", ["normal", "spike", "tiny", "huge"])
+def test_dense_small_tensors(fcs, ctx, orc, shape, J, D, nb, kind):
+    T = synth.gaussian(401, (nb,) + shape)
+    if kind == "spike":
+        T.reshape(nb, -1)[0, 0] = 3e7
+    elif kind != "normal":
+        T = (T.astype(np.float64) * (1e-30 if kind == "tiny" else 1e30)).astype(np.float32)
+    ho, so = orc.make_hashes(402, list(shape), J, D)
+    got = host(fcs.fcs_sketch_dense(ctx, cuda(T), J, cuda(ho), cuda(so), batched=True))
+    ref = _dense_ref(orc, T, J, ho, so)
+    assert_sketch_close(got, ref)
+    if kind == "spike":                  # the other bins keep their own accuracy
+        S = np.zeros_like(T[0])
+        S.reshape(-1)[0] = T.reshape(nb, -1)[0, 0]
+        keep = orc.fcs_dense(S.astype(np.float64), J, ho, so) == 0
+        for d in range(D):
+            r = ref[0, d][keep[d]]
+            if np.linalg.norm(r) > 0:
+                assert np.linalg.norm(got[0, d][keep[d]] - r) <= 1e-5 * np.linalg.norm(r)
+
+
+def test_dense_small_tensor_nan_and_bad_hash(fcs, ctx, orc):
+    shape, J, D = (9, 10, 12), [20, 30, 40], 3
+    T = synth.gaussian(403, (2,) + shape)
+    T[1, 4, 4, 4], T[1, 2, 3, 5] = np.nan, np.inf
+    ho, so = orc.make_hashes(404, list(shape), J, D)
+    bad = ho.copy()
+    bad[0, 3], bad[1, 9 + 2], bad[2, 19 + 7] = -1, 30, 1 << 29
+    ref = _dense_ref(orc, T, J, ho, so)
+    for d, (n, i) in enumerate([(0, 3), (1, 2), (2, 7)]):
+        Z = T.copy()
+        Z[(slice(None), *[slice(None)] * n, i)] = 0.0
+        ref[:, d] = _dense_ref(orc, Z, J, ho, so)[:, d]
+    got = host(fcs.fcs_sketch_dense(ctx, cuda(T), J, cuda(bad), cuda(so), batched=True))
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    fin = np.isfinite(ref)
+    assert np.array_equal(np.isfinite(got), fin)
+    assert np.linalg.norm(got[fin] - ref[fin]) <= 1e-5 * np.linalg.norm(ref[fin])
+
+
+@pytest.mark.parametrize("B,C,D,Jt", [(1, 1, 1, 1), (5, 3, 16, 31), (256, 10, 5, 178), (6, 130, 2, 33),
+                                      (700, 9, 3, 1000), (2000, 200, 2, 40)])
+def test_inner_products(fcs, ctx, B, C, D, Jt):
+    sa, sw = synth.gaussian(405, (B, D, Jt)), synth.gaussian(406, (C, D, Jt))
+    bias = synth.gaussian(407, (C,))
+    y, raw = fcs.fcs_sketch_inner(ctx, cuda(sa), cuda(sw), cuda(bias), raw=True)
+    ref = np.einsum("bdj,cdj->bcd", sa.astype(np.float64), sw.astype(np.float64))
+    tol = CONTRACT_RTOL * np.linalg.norm(sa, axis=2)[:, None, :] * np.linalg.norm(sw, axis=2)[None]
+    assert np.all(np.abs(host(raw) - ref) <= tol)
+    assert np.all(np.abs(host(y) - (np.median(ref, axis=2) + bias)) <= tol.max(axis=2) + 1e-6)
+    y2 = fcs.fcs_sketch_inner(ctx, cuda(sa), cuda(sw))
+    assert np.all(np.abs(host(y2) - np.median(ref, axis=2)) <= tol.max(axis=2))
