@@ -82,84 +82,174 @@ struct AlsArgs {
   int64_t I[kMaxN];
   float *F[kMaxN];       // [R][I_n] each
   float *Mt;             // [R][I_m]: in T_(m) columns (transposed), out the solution
+  float *gram;           // [N][R][R]: F_n F_n^T
   float *lambda;         // [R]
+  int in_smem;           // the solution fits shared memory
 };
 
-// One CTA: G = *_{n != m} F_n F_n^T, Cholesky G = L L^T, then for every
-// column i of M^T the solve G x = M^T[:, i]; row norms give lambda and the
-// normalised rows the new F_m.
-__global__ void __launch_bounds__(1024) als_update_kernel(AlsArgs a) {
+// g = V V^T for V [R][I]: one warp per pair of rows, two pairs at a time.
+// All threads of the block call it.
+__device__ __forceinline__ void gram_matrix(const float *V, int64_t I, int R, float *g) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const int pairs = R * (R + 1) / 2;
+  auto rows = [&](int p, int &r, int &q) {           // pair p of r >= q
+    r = int((sqrtf(8.f * float(p) + 1.f) - 1.f) * 0.5f);
+    while ((r + 1) * (r + 2) / 2 <= p) ++r;
+    while (r * (r + 1) / 2 > p) --r;
+    q = p - r * (r + 1) / 2;
+  };
+  for (int p = warp; p < pairs; p += 2 * warps) {
+    int r[2], q[2];
+    const int p1 = p + warps < pairs ? p + warps : p;
+    rows(p, r[0], q[0]);
+    rows(p1, r[1], q[1]);
+    float d0 = 0.f, d1 = 0.f;
+#pragma unroll 4
+    for (int64_t i = lane; i < I; i += 32) {
+      d0 = fmaf(V[r[0] * I + i], V[q[0] * I + i], d0);
+      d1 = fmaf(V[r[1] * I + i], V[q[1] * I + i], d1);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      d0 += __shfl_xor_sync(0xffffffffu, d0, o);
+      d1 += __shfl_xor_sync(0xffffffffu, d1, o);
+    }
+    if (lane == 0) {
+      g[r[0] * R + q[0]] = g[q[0] * R + r[0]] = d0;
+      g[r[1] * R + q[1]] = g[q[1] * R + r[1]] = d1;
+    }
+  }
+}
+
+// The Gram matrices of the starting factors, one block per mode.
+__global__ void __launch_bounds__(1024) als_gram_kernel(AlsArgs a) {
+  const int n = blockIdx.x;
+  gram_matrix(a.F[n], a.I[n], a.R, a.gram + n * a.R * a.R);
+}
+
+// One CTA: G = *_{n != m} F_n F_n^T from the Gram matrices, Cholesky G = L
+// L^T, then for every column i of M^T the solve G x = M^T[:, i]; row norms give
+// lambda and the normalised rows the new F_m, whose Gram matrix replaces the
+// old one.  Latency-bound (400 x 10: 50 us with the Gram products of whole
+// rows by one thread each, the factorisation by one thread and the solve's
+// vector in local memory; now 20 us): a warp factors, lane i holding row i, and
+// RM >= R lanes solve eight columns at a time, one element of each per lane (the
+// rows past R are those of the identity).
+constexpr int kUpdNT = 512;
+template <int RM>
+__global__ void __launch_bounds__(kUpdNT) als_update_kernel(AlsArgs a) {
+  extern __shared__ float xs[];               // [R][I_m] when it fits, else the solution stays in Mt
   __shared__ float G[kMaxRank][kMaxRank + 1];
-  __shared__ float nrm[kMaxRank];
-  const int R = a.R;
-  for (int p = threadIdx.x; p < R * R; p += blockDim.x) {
-    const int r = p / R, q = p % R;
-    float g = 1.f;
-    for (int n = 0; n < a.N; ++n) {
-      if (n == a.m) continue;
-      const float *fr = a.F[n] + int64_t(r) * a.I[n];
-      const float *fq = a.F[n] + int64_t(q) * a.I[n];
-      float dot = 0.f;
-      for (int64_t i = 0; i < a.I[n]; ++i) dot = fmaf(fr[i], fq[i], dot);
-      g *= dot;
+  __shared__ float sums[kUpdNT / RM][RM];
+  __shared__ float nrm[RM], inv[RM];
+  // x / g from inv = 1 / g, with the remainder added back (a division's slow
+  // path would cost the solve its registers)
+  auto quotient = [](float x, float g, float inv) {
+    const float q = x * inv;
+    return fmaf(fmaf(-q, g, x), inv, q);
+  };
+  const int R = a.R, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int p = tid; p < RM * RM; p += kUpdNT) {
+    const int r = p / RM, q = p % RM;
+    float g = r == q ? 1.f : 0.f;
+    if (r < R && q < R) {
+      g = 1.f;
+      for (int n = 0; n < a.N; ++n)
+        if (n != a.m) g *= a.gram[(n * R + r) * R + q];
     }
     G[r][q] = g;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // Cholesky in place (lower triangle); a non-positive pivot is lifted to a
-    // tiny multiple of the largest diagonal entry
-    float dmax = 0.f;
-    for (int r = 0; r < R; ++r) dmax = fmaxf(dmax, G[r][r]);
+  if (warp == 0) {
+    // right-looking, lower triangle; a non-positive pivot is lifted to a tiny
+    // multiple of the largest diagonal entry
+    float dmax = lane < R ? G[lane][lane] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
     for (int j = 0; j < R; ++j) {
       float v = G[j][j];
-      for (int k = 0; k < j; ++k) v -= G[j][k] * G[j][k];
       v = v > 1e-12f * dmax ? v : 1e-12f * dmax + 1e-30f;
       const float ljj = sqrtf(v);
-      G[j][j] = ljj;
-      for (int i = j + 1; i < R; ++i) {
-        float w = G[i][j];
-        for (int k = 0; k < j; ++k) w -= G[i][k] * G[j][k];
-        G[i][j] = w / ljj;
+      __syncwarp();
+      if (lane == j) G[j][j] = ljj;
+      float lij = 0.f;
+      if (lane > j && lane < R) {
+        lij = G[lane][j] / ljj;
+        G[lane][j] = lij;
+      }
+      __syncwarp();
+      if (lane > j && lane < R)
+        for (int k = j + 1; k <= lane; ++k) G[lane][k] -= lij * G[k][j];
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  if (tid < RM) inv[tid] = 1.f / G[tid][tid];
+  __syncthreads();
+  // the solves: lane r of a group of RM holds element r of Q columns, row r
+  // and column r of L
+  const int64_t Im = a.I[a.m];
+  float *X = a.in_smem ? xs : a.Mt;
+  constexpr int Q = 8, GROUPS = kUpdNT / RM;
+  const int r = tid & (RM - 1);
+  float row[RM], colm[RM];
+#pragma unroll
+  for (int k = 0; k < RM; ++k) {
+    row[k] = G[r][k];
+    colm[k] = G[k][r];
+  }
+  const float dg = G[r][r], iv = inv[r];
+  float ss = 0.f;
+  for (int64_t i0 = int64_t(tid / RM) * Q; i0 - int64_t(tid / RM) * Q < Im; i0 += GROUPS * Q) {
+    float x[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      x[q] = r < R && i0 + q < Im ? a.Mt[int64_t(r) * Im + i0 + q] : 0.f;
+#pragma unroll
+    for (int j = 0; j < RM; ++j) {            // L y = b
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const float y = quotient(x[q], dg, iv);
+        const float t = __shfl_sync(0xffffffffu, y, j, RM);
+        x[q] = r == j ? y : r > j ? x[q] - row[j] * t : x[q];
       }
     }
-  }
-  __syncthreads();
-  const int64_t Im = a.I[a.m];
-  for (int64_t i = threadIdx.x; i < Im; i += blockDim.x) {
-    float x[kMaxRank];
-    for (int r = 0; r < R; ++r) x[r] = a.Mt[int64_t(r) * Im + i];
-    for (int r = 0; r < R; ++r) {             // L y = b
-      float v = x[r];
-      for (int k = 0; k < r; ++k) v -= G[r][k] * x[k];
-      x[r] = v / G[r][r];
-    }
-    for (int r = R - 1; r >= 0; --r) {        // L^T x = y
-      float v = x[r];
-      for (int k = r + 1; k < R; ++k) v -= G[k][r] * x[k];
-      x[r] = v / G[r][r];
-    }
-    for (int r = 0; r < R; ++r) a.Mt[int64_t(r) * Im + i] = x[r];
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int r = warp; r < R; r += blockDim.x >> 5) {
-    float ss = 0.f;
-    for (int64_t i = lane; i < Im; i += 32) {
-      const float v = a.Mt[int64_t(r) * Im + i];
-      ss += v * v;
+#pragma unroll
+    for (int j = RM - 1; j >= 0; --j) {       // L^T x = y
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const float y = quotient(x[q], dg, iv);
+        const float t = __shfl_sync(0xffffffffu, y, j, RM);
+        x[q] = r == j ? y : r < j ? x[q] - colm[j] * t : x[q];
+      }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) nrm[r] = sqrtf(ss);
+    for (int q = 0; q < Q; ++q) {
+      ss = fmaf(x[q], x[q], ss);
+      if (r < R && i0 + q < Im) X[int64_t(r) * Im + i0 + q] = x[q];
+    }
+  }
+  sums[tid / RM][r] = ss;
+  __syncthreads();
+  if (tid < RM) {
+    float t = 0.f;
+    for (int w = 0; w < GROUPS; ++w) t += sums[w][tid];
+    t = sqrtf(t);
+    nrm[tid] = t;
+    if (tid < R) a.lambda[tid] = t;
   }
   __syncthreads();
-  for (int64_t e = threadIdx.x; e < int64_t(R) * Im; e += blockDim.x) {
-    const int r = int(e / Im);
-    const float w = nrm[r];
-    a.F[a.m][e] = w > 0.f ? a.Mt[e] / w : 0.f;
+  float *F = a.F[a.m];
+  for (int64_t i = tid; i < Im; i += kUpdNT) {
+#pragma unroll
+    for (int k = 0; k < RM; ++k) {
+      if (k >= R) break;
+      const int64_t e = int64_t(k) * Im + i;
+      X[e] = F[e] = nrm[k] > 0.f ? X[e] / nrm[k] : 0.f;
+    }
   }
-  if (threadIdx.x < R) a.lambda[threadIdx.x] = nrm[threadIdx.x];
+  __syncthreads();
+  gram_matrix(X, Im, R, a.gram + a.m * R * R);
 }
 
 // Turns the spectrum cache on for the duration of a call and restores it.
@@ -281,7 +371,8 @@ extern "C" int fcs_als(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t
     imax = std::max<int64_t>(imax, host_I[n]);
   }
   DeviceGuard g(ctx->device);
-  rc = ensure_algo(ctx, sizeof(float) * size_t(R) * size_t(imax));
+  const size_t b_mt = (sizeof(float) * size_t(R) * size_t(imax) + 255) & ~size_t(255);
+  rc = ensure_algo(ctx, b_mt + sizeof(float) * size_t(N) * R * R);
   if (rc) return rc;
   float *Mt = static_cast<float *>(ctx->algo);
   CacheScope cache(ctx);
@@ -295,7 +386,13 @@ extern "C" int fcs_als(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t
     a.F[n] = host_F[n];
   }
   a.Mt = Mt;
+  a.gram = reinterpret_cast<float *>(static_cast<char *>(ctx->algo) + b_mt);
   a.lambda = lambda;
+  if (n_iter > 0) {
+    als_gram_kernel<<<N, 1024, 0, ctx->stream>>>(a);
+    rc = check_cuda(ctx, cudaGetLastError(), "als_gram_kernel");
+    if (rc) return rc;
+  }
   for (int it = 0; it < n_iter; ++it) {
     for (int mm = 0; mm < N; ++mm) {
       for (int n = 0; n < N; ++n) vv[n] = n == mm ? nullptr : host_F[n];
@@ -303,7 +400,15 @@ extern "C" int fcs_als(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t
                         s, ldh, Mt, nullptr);
       if (rc) return rc;
       a.m = mm;
-      als_update_kernel<<<1, 1024, 0, ctx->stream>>>(a);
+      const size_t xb = sizeof(float) * size_t(R) * size_t(host_I[mm]);
+      a.in_smem = xb <= 40 * 1024;
+      const size_t xsm = a.in_smem ? xb : 0;
+      if (R <= 8)
+        als_update_kernel<8><<<1, kUpdNT, xsm, ctx->stream>>>(a);
+      else if (R <= 16)
+        als_update_kernel<16><<<1, kUpdNT, xsm, ctx->stream>>>(a);
+      else
+        als_update_kernel<32><<<1, kUpdNT, xsm, ctx->stream>>>(a);
       rc = check_cuda(ctx, cudaGetLastError(), "als_update_kernel");
       if (rc) return rc;
     }

@@ -88,3 +88,22 @@ def test_inner_products(fcs, ctx, B, C, D, Jt):
     assert np.all(np.abs(host(y) - (np.median(ref, axis=2) + bias)) <= tol.max(axis=2) + 1e-6)
     y2 = fcs.fcs_sketch_inner(ctx, cuda(sa), cuda(sw))
     assert np.all(np.abs(host(y2) - np.median(ref, axis=2)) <= tol.max(axis=2))
+
+
+@pytest.mark.parametrize("R", [1, 2, 8, 9, 16, 17, 32])
+def test_als_update_ranks(fcs, ctx, orc, R):
+    """One sweep from orthogonal-ish factors: same factors as the oracle's
+    loop (cond(G) stays below 10, so the contraction bar carries over)."""
+    import oracle.algorithms as alg
+    I, J, D = [90, 70, 110], [3000, 2000, 2500], 3
+    U, lam = synth.cp_factors(408, I, R)
+    ho, so = orc.make_hashes(409, I, J, D)
+    hg, sg = cuda(ho), cuda(so)
+    fT = fcs.fcs_sketch_cp(ctx, [cuda(u) for u in U], cuda(lam), J, hg, sg)
+    init = [synth.orthonormal_columns(410 + n, i, R).T.astype(np.float32).copy() for n, i in enumerate(I)]
+    F = [cuda(x.copy()) for x in init]
+    lam_g = host(fcs.fcs_als(ctx, fT, I, J, hg, sg, F, 1))
+    Fref, lref = alg.als(host(fT).astype(np.float64), I, J, ho, so, R, 1, init)
+    np.testing.assert_allclose(lam_g, lref, rtol=3e-3)
+    for f, fr in zip(F, Fref):
+        np.testing.assert_allclose(host(f), fr, atol=3e-3)
