@@ -13,7 +13,11 @@
 // Kernels: (1) the half spectra of the D sketches of T; (2) one CTA per
 // (batch item, sketch) that builds each needed Count Sketch in shared memory,
 // transforms it and folds it into the per-thread spectrum product, then either
-// reduces the Parseval sum or runs the inverse FFT and gathers; (3) the median.
+// reduces the Parseval sum or runs the inverse FFT and gathers; (3) the median
+// (of both results in one launch).  (2) runs on the slot FFT of fcs_fft.cuh
+// and, for large batches at P = 16384, on the row-pair engine of fcs_pair.cuh.
+// Each kernel is launched so that it may start before the one before has
+// ended and waits where it first reads what that one wrote.
 //
 // With fcs_cache_spectra enabled, the spectra of (1) are kept in a
 // per-context cache keyed by the sketch pointer and shape, so repeated
@@ -22,7 +26,7 @@
 // entries of the buffers they overwrite.
 #include <vector>
 
-#include "fcs_fft.cuh"
+#include "fcs_pair.cuh"
 
 struct fcs_spec_cache {
   struct Entry {
@@ -147,6 +151,7 @@ __global__ void __launch_bounds__(NT) spectrum_kernel(const float *__restrict__ 
   float2 *tws = reinterpret_cast<float2 *>(smem + Lay::kTw);
   float *A = reinterpret_cast<float *>(smem + Lay::kA);
   const float *xd = x + blockIdx.x * ld;
+  griddep_launch();
   fill_twiddles<LOG2M, NT>(tws, tw);
   float2 *lps = reinterpret_cast<float2 *>(smem + Lay::kLp);
   LastPassTwShared<LOG2M, NT>::fill(lps, tw);
@@ -202,21 +207,26 @@ __global__ void __launch_bounds__(NT) contract_kernel(ContractArgs a,
   for (int e = tid; e < sb / 4; e += NT)
     reinterpret_cast<float4 *>(A)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
 
-  // spectrum of FCS_d(T) in this thread's slots, and the running product
-  float2 F[EPS][2][RL], p[EPS][2][RL], X[EPS][2][RL];
+  // the running product in this thread's slots; the spectrum of FCS_d(T) in
+  // the same slots (the q = 0 slot packs two reals) is read where it is first
+  // used, since spectrum_kernel may still be running before
+  float2 p[EPS][2][RL], X[EPS][2][RL];
+  auto spec_at = [&](int e, int bb, int r) {
+    const bool live = LPs::SLOTS % NT == 0 || tid + e * NT < LPs::SLOTS;
+    const int q = live ? last_pass_index<LOG2M, NT>(e, bb, r) : 1;
+    return live ? (q == 0 ? make_float2(__ldcg(&sd[0].x), __ldcg(&sd[M].x)) : __ldcg(sd + q))
+                : make_float2(0.f, 0.f);
+  };
+  auto spec_to_p = [&] {
+    griddep_wait();
 #pragma unroll
-  for (int e = 0; e < EPS; ++e)
+    for (int e = 0; e < EPS; ++e)
 #pragma unroll
-    for (int bb = 0; bb < 2; ++bb)
+      for (int bb = 0; bb < 2; ++bb)
 #pragma unroll
-      for (int r = 0; r < RL; ++r) {
-        const bool live = LPs::SLOTS % NT == 0 || tid + e * NT < LPs::SLOTS;
-        const int q = live ? last_pass_index<LOG2M, NT>(e, bb, r) : 1;
-        F[e][bb][r] = live ? (q == 0 ? make_float2(sd[0].x, sd[M].x) : sd[q])
-                           : make_float2(0.f, 0.f);
-        // multiplicative identity; the q = 0 slot packs two reals
-        p[e][bb][r] = all ? make_float2(1.f, q == 0 ? 1.f : 0.f) : F[e][bb][r];
-      }
+        for (int r = 0; r < RL; ++r) p[e][bb][r] = spec_at(e, bb, r);
+  };
+  bool first = true;
 
   for (int n = 0; n < a.m.N; ++n) {
     if (!all && n == a.free_mode) continue;
@@ -231,6 +241,7 @@ __global__ void __launch_bounds__(NT) contract_kernel(ContractArgs a,
       if (unsigned(hb) < unsigned(sb)) atomicAdd(A + hb, v);
     }
     rfft_to_slots<LOG2M, NT>(A, sb, B, tws, ltw, X);
+    if (first && !all) spec_to_p();
 #pragma unroll
     for (int e = 0; e < EPS; ++e)
 #pragma unroll
@@ -238,12 +249,19 @@ __global__ void __launch_bounds__(NT) contract_kernel(ContractArgs a,
 #pragma unroll
         for (int r = 0; r < RL; ++r) {
           const bool packed = bb == 0 && r == 0 && tid + e * NT == 0;
-          p[e][bb][r] = all ? slot_mul(p[e][bb][r], X[e][bb][r], packed)
-                            : slot_mulconj(p[e][bb][r], X[e][bb][r], packed);
+          if (all && first)
+            p[e][bb][r] = X[e][bb][r];
+          else
+            p[e][bb][r] = all ? slot_mul(p[e][bb][r], X[e][bb][r], packed)
+                              : slot_mulconj(p[e][bb][r], X[e][bb][r], packed);
         }
+    first = false;
   }
+  if (first && !all) spec_to_p();                 // FREE of order 1
+  griddep_launch();
 
   if (all) {
+    griddep_wait();
     // sum_{k<P} conj(F_T[k]) Y[k]: the packed q = 0 slot holds the real bins
     // 0 and M (weight 1); every other bin q in (0, M) appears twice
     float part = 0.f;
@@ -255,7 +273,8 @@ __global__ void __launch_bounds__(NT) contract_kernel(ContractArgs a,
 #pragma unroll
         for (int r = 0; r < RL; ++r) {
           const bool packed = bb == 0 && r == 0 && tid + e * NT == 0;
-          const float dot = F[e][bb][r].x * p[e][bb][r].x + F[e][bb][r].y * p[e][bb][r].y;
+          const float2 f = spec_at(e, bb, r);
+          const float dot = f.x * p[e][bb][r].x + f.y * p[e][bb][r].y;
           part += packed ? dot : 2.f * dot;
         }
     }
@@ -330,21 +349,270 @@ __global__ void __launch_bounds__(NT) contract_kernel(ContractArgs a,
   }
 }
 
+// ---------------------------------------------------------------- P = 16384
+// contract_kernel on the row-pair engine: one CTA per (item b, sketch d), two
+// to an SM (contract_kernel's registers and buffers leave room for one).  The
+// running product is in tensor memory between transforms; every forward
+// transform leaves twice the spectrum, so results scale by 2^-transforms.
+template <int NR>
+__global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
+    contract_pair_kernel(ContractArgs a, const float2 *__restrict__ tw) {
+  using Geo = pfft::Geo<NR>;
+  using Lay = pfft::Smem<NR>;
+  constexpr int NT = Geo::NT, M = Geo::M, HALF = M / 2, H = Geo::H;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ uint32_t slot;
+  __shared__ float red[NT / 32];
+  float4 *B = reinterpret_cast<float4 *>(smem + Lay::kB);
+  const float2 *t0 = reinterpret_cast<float2 *>(smem + Lay::kT0);
+  const float2 *t1 = reinterpret_cast<float2 *>(smem + Lay::kT1);
+  const float2 *t2 = reinterpret_cast<float2 *>(smem + Lay::kT2);
+  const float2 *t3 = reinterpret_cast<float2 *>(smem + Lay::kT3);
+  float4 *A4 = reinterpret_cast<float4 *>(smem + Lay::kA);
+  float *A = reinterpret_cast<float *>(A4);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t b = blockIdx.x;
+  const int d = blockIdx.y, N = a.m.N, sb = a.sb;
+  const int ra = (sb + 2 * NR - 1) / (2 * NR);
+  const bool all = a.kind == FCS_CONTRACT_ALL, both = a.kind == kBoth;
+  const float2 *sd = a.spec + d * int64_t(M + 1);
+  const uint32_t tm = pfft::tmem_alloc<NR>(&slot);
+  const uint32_t tp = pfft::tmem_mine<NR>(tm);
+  const bool w0 = warp == Geo::WARPS - 1;            // the warp that has column 0
+  pfft::fill_twiddles<NR>(smem, tw);
+  for (int e = tid; e < H * ra; e += NT) A4[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
+  // mode of transform k: those of the product in order, the free one last
+  const int last = all ? N - 1 : both ? N - 1 : N - 2;
+  auto mode_of = [&](int k) {
+    return all ? k : k == N - 1 ? a.free_mode : k < a.free_mode ? k : k + 1;
+  };
+  auto scatter = [&](int n) {
+    const int32_t *hn = a.h + d * a.m.ldh + a.m.off[n];
+    const int8_t *sn = a.s + d * a.m.ldh + a.m.off[n];
+    const float *vn = a.vec[n] + b * a.m.I[n];
+#pragma unroll 4
+    for (int64_t i = tid; i < a.m.I[n]; i += NT) {
+      const float v = __ldg(vn + i);
+      const int hb = __ldg(hn + i);
+      if (unsigned(hb) < unsigned(sb))
+        atomicAdd(A + pfft::a_index<NR>(hb, ra), __ldg(sn + i) < 0 ? -v : v);
+    }
+  };
+  if (last >= 0) scatter(mode_of(0));
+  __syncthreads();
+  float2 p0 = make_float2(1.f, lane == 0 ? 1.f : 0.f);   // column 0's product
+  const int i0 = lane & (NR - 1);
+  float2 f0 = make_float2(0.f, 0.f);                 // column 0 of FCS_d(T)'s spectrum
+  auto spec_wait = [&] {
+    griddep_wait();
+    f0 = i0 ? __ldcg(sd + 512 * i0) : make_float2(__ldcg(&sd[0].x), __ldcg(&sd[M].x));
+    if (!all) p0 = f0;
+  };
+  float part = 0.f;                                  // of the Parseval sum
+  // spectrum of FCS_d(T) at the bins of value i (0 .. 2H - 1) of pair c
+  auto spec_at = [&](int c, int i) {
+    const int bb = i < H ? 0 : 1, k = i < H ? i : (2 * H - i) % H;
+    const float2 u = __ldcg(sd + pfft::bin_of<NR>(c, bb, k, 0));
+    const float2 v = __ldcg(sd + pfft::bin_of<NR>(c, bb, k, 1));
+    return pfft::C2{pfft::pk(u.x, v.x), pfft::pk(u.y, v.y)};
+  };
+  for (int k = 0; k <= last; ++k) {
+    pfft::scatter_row_step<Geo::RPW, Geo::PAD>(A4 + warp * ra, Geo::WARPS * ra, ra,
+                                               B + warp * Geo::RS, Geo::WARPS * Geo::RS, t0, t1);
+    __syncthreads();
+    const bool early = tid < NT / 2;
+    if (k < last && early) scatter(mode_of(k + 1));
+    // dot: the Parseval sum over this transform (no product is kept)
+    const bool dot = (all || both) && k == N - 1;
+    if (k == (all ? N - 1 : 0)) spec_wait();         // first use of the spectrum
+    if (w0) {
+      const float2 x = pfft::column0<NR>(B, t3);
+      if (dot) {
+        const float2 y = all ? slot_mul(p0, x, lane == 0) : x;
+        const float2 g = all ? f0 : p0;
+        if (lane < NR) part += (lane ? 2.f : 1.f) * (g.x * y.x + g.y * y.y);
+      } else {
+        p0 = all ? slot_mul(p0, x, lane == 0) : slot_mulconj(p0, x, lane == 0);
+      }
+    }
+#pragma unroll 1
+    for (int c = 0; c < Geo::NCP; ++c) {
+      pfft::C2 xa[H], xc[H];
+      pfft::column_step<NR>(B, t2, c, xa, xc);
+      pfft::unpack<NR>(t2, c, xa, xc);
+      const uint32_t o = tp + uint32_t(c) * (8 * H);
+      __syncwarp();                                  // tensor-memory accesses are warp-wide
+#pragma unroll
+      for (int g = 0; g < 2 * H; g += 4) {
+        pfft::Tm16 x;
+        const bool load = k > 0;
+        if (load) {
+          pfft::tmem_ld16(o + 4 * g, x);
+          pfft::tmem_wait_ld(x);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          pfft::C2 v = g < H ? xa[g + i] : xc[g - H + i];
+          if (all) {
+            if (load) v = pfft::cmul(pfft::tm_get(x, i), v);
+          } else if (!dot) {
+            const pfft::C2 y = load ? pfft::tm_get(x, i) : spec_at(c, g + i);
+            v = pfft::cmul3(y, v.re, pfft::neg2(v.im), v.im);      // y conj(v)
+          }
+          if (dot) {
+            const pfft::C2 f = all || !load ? spec_at(c, g + i) : pfft::tm_get(x, i);
+            const pfft::f2x t = pfft::fma2(f.re, v.re, pfft::mul2(f.im, v.im));
+            // (u = 256: its second column repeats the first)
+            if (g < H || tid + c * NT != 255) part += 2.f * (pfft::lo(t) + pfft::hi(t));
+          } else {
+            pfft::tm_set(x, i, v);
+          }
+        }
+        __syncwarp();
+        if (!dot) pfft::tmem_st16(o + 4 * g, x);
+      }
+    }
+    pfft::tmem_wait_st();
+    if (k < last && !early) scatter(mode_of(k + 1));
+    __syncthreads();
+  }
+  if (last < 0) spec_wait();                         // FREE of order 1
+  griddep_launch();
+  if (all || both) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if (lane == 0) red[warp] = part;
+    __syncthreads();
+    if (tid == 0) {
+      float t = 0.f;
+      for (int w = 0; w < NT / 32; ++w) t += red[w];
+      (all ? a.raw : a.raw_all)[b * a.D + d] = t / (float(2 * M) * float(1 << N));
+    }
+  }
+  if (!all) {
+    // FREE: the conj-packed product into B (every pair (q, M - q) is a
+    // thread's), an inverse transform, then the gather at h_m(i)
+    float *Bf = reinterpret_cast<float *>(B);
+    auto put = [&](int m, float2 z) {
+      float *p = Bf + pfft::b_index<NR>(m);
+      p[0] = z.x;
+      p[2] = z.y;
+    };
+#pragma unroll 1
+    for (int c = 0; c < Geo::NCP; ++c) {
+      const uint32_t o = tp + uint32_t(c) * (8 * H);
+      pfft::Tm16 x[H / 2];
+      __syncwarp();
+      if (N > 1) {
+#pragma unroll
+        for (int g = 0; g < H / 2; ++g) pfft::tmem_ld16(o + 16 * g, x[g]);
+#pragma unroll
+        for (int g = 0; g < H / 2; ++g) pfft::tmem_wait_ld(x[g]);
+      } else {                                       // no other mode: the sketch itself
+#pragma unroll
+        for (int i = 0; i < 2 * H; ++i) pfft::tm_set(x[i / 4], i % 4, spec_at(c, i));
+      }
+      const float2 wP = t2[Geo::LNR * 256 + tid + c * NT];
+      const int u = tid + 1 + c * NT;
+#pragma unroll
+      for (int K = 0; K < H; ++K) {
+        const int kc = H + (H - K) % H;
+        const pfft::C2 va = pfft::tm_get(x[K / 4], K % 4), vc = pfft::tm_get(x[kc / 4], kc % 4);
+        const float2 w = K == 0 ? wP : cmul(wP, unit64(K * 32 / NR));
+        float2 cq, cm;
+        const int q = u + 512 * K;
+        pack_pair_conj_values_w(q, make_float2(pfft::lo(va.re), pfft::lo(va.im)),
+                                make_float2(pfft::lo(vc.re), pfft::lo(vc.im)), w, cq, cm);
+        put(q, cq);
+        put(M - q, cm);
+        const int r = q + HALF;
+        pack_pair_conj_values_w(r, make_float2(pfft::hi(va.re), pfft::hi(va.im)),
+                                make_float2(pfft::hi(vc.re), pfft::hi(vc.im)),
+                                make_float2(w.y, -w.x), cq, cm);
+        put(r, cq);
+        put(M - r, cm);
+      }
+    }
+    if (w0) {
+      // lane i: X[512 i], paired with X[512 (NR - i)]
+      float2 y;
+      y.x = __shfl_sync(0xffffffffu, p0.x, (NR - i0) & (NR - 1));
+      y.y = __shfl_sync(0xffffffffu, p0.y, (NR - i0) & (NR - 1));
+      if (lane < NR) {
+        float2 cq, cm;
+        pack_pair_conj_values_w(lane, p0, y, t3[lane], cq, cm);
+        put(512 * lane, lane == NR / 2 ? p0 : cq);
+      }
+    }
+    __syncthreads();
+    pfft::row_step<32, true, Geo::RPW, Geo::PAD>(B + warp * Geo::RS, Geo::WARPS * Geo::RS, 512,
+                                                 B + warp * Geo::RS, Geo::WARPS * Geo::RS, t0, t1);
+    __syncthreads();
+    // z[m] in natural order over B once every column has been read
+    float2 *Z = reinterpret_cast<float2 *>(B);
+    pfft::C2 xa[Geo::NCP][H], xc[Geo::NCP][H];
+#pragma unroll
+    for (int c = 0; c < Geo::NCP; ++c) pfft::column_step<NR>(B, t2, c, xa[c], xc[c]);
+    float2 z0 = make_float2(0.f, 0.f);
+    if (w0) z0 = pfft::column0_complex<NR>(B, t3);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < Geo::NCP; ++c) {
+      const int u = tid + 1 + c * NT, uc = 512 - u;
+#pragma unroll
+      for (int k = 0; k < H; ++k) {
+        Z[u + 512 * k] = make_float2(pfft::lo(xa[c][k].re), pfft::lo(xa[c][k].im));
+        Z[u + 512 * (k + H)] = make_float2(pfft::hi(xa[c][k].re), pfft::hi(xa[c][k].im));
+        const int ql = (k == 0 ? NR - 1 : k + H - 1), qh = (k == 0 ? H - 1 : k - 1);
+        Z[uc + 512 * ql] = make_float2(pfft::lo(xc[c][k].re), pfft::lo(xc[c][k].im));
+        Z[uc + 512 * qh] = make_float2(pfft::hi(xc[c][k].re), pfft::hi(xc[c][k].im));
+      }
+    }
+    if (w0 && lane < NR) Z[512 * lane] = z0;
+    __syncthreads();
+    const int m = a.free_mode;
+    const int32_t *hm = a.h + d * a.m.ldh + a.m.off[m];
+    const int8_t *sm = a.s + d * a.m.ldh + a.m.off[m];
+    const int64_t Im = a.m.I[m];
+    float *rawbd = a.raw + (b * a.D + d) * Im;
+    const float sc = 1.0f / (float(M) * float(1 << (N - 1)));
+    for (int64_t i = tid; i < Im; i += NT) {
+      const int pz = __ldg(hm + i);
+      const float v = unsigned(pz) < unsigned(2 * M) ? Bf[pz] : __int_as_float(0x7fc00000);
+      const float z = (pz & 1) ? -v * sc : v * sc;
+      rawbd[i] = __ldg(sm + i) < 0 ? -z : z;
+    }
+  }
+  pfft::tmem_free<NR>(tm);
+}
+
+// raw [B][D][width] -> out [B][width] and, when out2 is given, raw2 [B][D] ->
+// out2 [B].
 template <int D>
-__global__ void median_kernel(const float *__restrict__ raw, int64_t B, int64_t width,
-                              float *__restrict__ out) {
-  // raw [B][D][width] -> out [B][width]
+__global__ void median_kernel(const float *raw, int64_t B, int64_t width, float *out,
+                              const float *raw2, float *out2) {
   const int64_t total = B * width;
-  for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total;
+  griddep_wait();
+  for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total + (out2 ? B : 0);
        t += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t b = t / width, i = t - b * width;
+    const bool one = t < total;
+    const int64_t w = one ? width : 1, e = one ? t : t - total;
+    const int64_t b = e / w, i = e - b * w;
+    const float *src = one ? raw : raw2;
     float v[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) v[d] = raw[(b * D + d) * width + i];
-    out[t] = median_inplace<D>(v);
+    for (int d = 0; d < D; ++d) v[d] = __ldcg(src + (b * D + d) * w + i);
+    (one ? out : out2)[e] = median_inplace<D>(v);
   }
 }
 
+// P = 16384 has two kernels.  With more CTAs than SMs the row-pair engine is
+// the faster one (order 3, 400^3, D = 5, both results: 64 items 64 us for 74,
+// 1024 items 524 for 709); with fewer, one 512-thread CTA of contract_kernel
+// has the shorter chain (10 items 33 us for 36).  At P = 8192 contract_kernel
+// is as fast in large batches (1024 items 339 us for 324) and faster in small
+// ones (10 items 23.5 us for 33.6).
 template <int LOG2M>
 int launch_contract(fcs_ctx *ctx, ContractArgs &a, int64_t Jt, bool need_spec,
                     cudaEvent_t spec_ready) {
@@ -355,10 +623,9 @@ int launch_contract(fcs_ctx *ctx, ContractArgs &a, int64_t Jt, bool need_spec,
   auto k1 = spectrum_kernel<LOG2M, NT>;
   auto k2 = contract_kernel<LOG2M, NT>;
   cudaError_t e = cudaSuccess;
-  if (smem1 > 48 * 1024)
-    e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem1));
+  if (smem1 > 48 * 1024) e = allow_smem(reinterpret_cast<const void *>(k1), smem1);
   if (e == cudaSuccess && smem2 > 48 * 1024)
-    e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem2));
+    e = allow_smem(reinterpret_cast<const void *>(k2), smem2);
   if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(contract)");
   if (need_spec) {
     k1<<<a.D, NT, smem1, ctx->stream>>>(a.fcsT, Jt, Jt, sb_spec, a.spec, ctx->twiddle);
@@ -369,19 +636,41 @@ int launch_contract(fcs_ctx *ctx, ContractArgs &a, int64_t Jt, bool need_spec,
       if (rc) return rc;
     }
   }
-  k2<<<dim3(unsigned(a.B), unsigned(a.D)), NT, smem2, ctx->stream>>>(a, ctx->twiddle);
-  return check_cuda(ctx, cudaGetLastError(), "contract_kernel");
+  // Directly behind spectrum_kernel the transforms of the vectors start while
+  // the D CTAs of the spectra still run (9 us of a chain of 42 at 64 items, P =
+  // 8192, D = 5): the kernel waits where it first reads them.
+  const bool overlap = need_spec && !spec_ready;
+  const dim3 grid{unsigned(a.B), unsigned(a.D)};
+  if constexpr (LOG2M == 13) {
+    if (a.B * a.D > ctx->sm_count) {
+      constexpr int NR = 16;
+      const size_t smem3 = pfft::Smem<NR>::bytes((a.sb + 2 * NR - 1) / (2 * NR));
+      auto k3 = contract_pair_kernel<NR>;
+      e = allow_smem(reinterpret_cast<const void *>(k3), smem3);
+      if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(contract)");
+      return check_cuda(ctx, launch_dep(k3, grid, pfft::Geo<NR>::NT, smem3, ctx->stream, overlap,
+                                        a, ctx->twiddle),
+                        "contract_pair_kernel");
+    }
+  }
+  return check_cuda(ctx, launch_dep(k2, grid, NT, smem2, ctx->stream, overlap, a, ctx->twiddle),
+                    "contract_kernel");
 }
 
-int launch_median(fcs_ctx *ctx, int D, const float *raw, int64_t B, int64_t width,
-                  float *out) {
-  const int64_t total = B * width;
+// dep: the kernel before on the stream is the one that writes raw and raw2
+int launch_median(fcs_ctx *ctx, int D, const float *raw, int64_t B, int64_t width, float *out,
+                  const float *raw2, float *out2, bool dep) {
+  const int64_t total = B * width + (out2 ? B : 0);
+  cudaError_t e = cudaSuccess;
   int blocks = int((total + 255) / 256);
   if (blocks > 4096) blocks = 4096;
   if (blocks < 1) blocks = 1;
   switch (D) {
 #define FCS_MED_CASE(K) \
-  case K: median_kernel<K><<<blocks, 256, 0, ctx->stream>>>(raw, B, width, out); break;
+  case K:                                                                                   \
+    e = launch_dep(median_kernel<K>, blocks, 256, 0, ctx->stream, dep, raw, B, width, out, \
+                   raw2, out2);                                                            \
+    break;
     FCS_MED_CASE(1) FCS_MED_CASE(2) FCS_MED_CASE(3) FCS_MED_CASE(4) FCS_MED_CASE(5)
     FCS_MED_CASE(6) FCS_MED_CASE(7) FCS_MED_CASE(8) FCS_MED_CASE(9) FCS_MED_CASE(10)
     FCS_MED_CASE(11) FCS_MED_CASE(12) FCS_MED_CASE(13) FCS_MED_CASE(14) FCS_MED_CASE(15)
@@ -390,7 +679,7 @@ int launch_median(fcs_ctx *ctx, int D, const float *raw, int64_t B, int64_t widt
     default:
       return set_error(ctx, FCS_EINVAL, "D=%d outside [1,16]", D);
   }
-  return check_cuda(ctx, cudaGetLastError(), "median_kernel");
+  return check_cuda(ctx, e, "median_kernel");
 }
 
 }  // namespace
@@ -542,15 +831,14 @@ int contract_call(fcs_ctx *ctx, int kind, int free_mode, int N, const int64_t *h
     if (ent && !hit) ent->stale = true;          // never computed
     return rc;
   }
+  rc = launch_median(ctx, D, a.raw, B, width, out_median, a.raw_all, both ? out_all : nullptr,
+                     !big);
   if (ent) {
-    rc = check_cuda(ctx, cudaEventRecord(ent->used, ctx->stream), "cudaEventRecord");
-    if (rc) return rc;
+    const int re =
+        check_cuda(ctx, cudaEventRecord(ent->used, ctx->stream), "cudaEventRecord");
+    if (!rc) rc = re;
   }
-  if (both) {
-    rc = launch_median(ctx, D, a.raw_all, B, 1, out_all);
-    if (rc) return rc;
-  }
-  return launch_median(ctx, D, a.raw, B, width, out_median);
+  return rc;
 }
 
 }  // namespace

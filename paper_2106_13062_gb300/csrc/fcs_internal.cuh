@@ -99,6 +99,35 @@ inline cudaError_t allow_smem(const void *kern, size_t bytes) {
                               int(bytes > kMaxDynSmem ? bytes : kMaxDynSmem));
 }
 
+// Programmatic dependent launch: with dep, the kernel may start as soon as
+// every CTA of the kernel before it on the stream has called griddep_launch()
+// or ended, and has to call griddep_wait() before it touches anything that
+// kernel reads or writes in global memory.  griddep_wait() returns once the
+// kernel before is complete and its writes are visible; every CTA of a kernel
+// launched with dep calls it, so that kernels end in stream order.  Without dep
+// both calls do nothing.
+__device__ __forceinline__ void griddep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void griddep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                       cudaStream_t stream, bool dep, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = dep ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 inline int ilog2_ceil(int64_t x) {
   int l = 0;
   while ((int64_t(1) << l) < x) ++l;

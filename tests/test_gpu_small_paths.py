@@ -107,3 +107,41 @@ def test_als_update_ranks(fcs, ctx, orc, R):
     np.testing.assert_allclose(lam_g, lref, rtol=3e-3)
     for f, fr in zip(F, Fref):
         np.testing.assert_allclose(host(f), fr, atol=3e-3)
+
+
+@pytest.mark.parametrize("kind", ["all", "free", "both"])
+@pytest.mark.parametrize("I,J,D,B,m", [
+    ([300], [8192], 2, 3, 0), ([300], [16384], 1, 160, 0), ([40, 700], [4097, 4097], 3, 55, 1),
+    ([50, 60, 70], [2049, 2900, 3000], 4, 5, 0), ([50, 60, 70], [5461, 5462, 5461], 2, 80, 2),
+    ([30, 20, 25, 35], [3000, 2500, 100, 2600], 5, 2, 1), ([1200, 20], [9000, 7000], 1, 155, 0),
+    ([30, 20, 25, 35], [4000, 2500, 100, 2600], 4, 40, 1), ([60, 90], [8000, 8385], 2, 3, 0),
+])
+def test_contract_long(fcs, ctx, orc, I, J, D, B, m, kind):
+    """P = 8192 and 16384 at the ends of their ranges, every kind, in few and
+    in more items than SMs (the row-pair engine at P = 16384), against the
+    FP64 contraction of the same sketch."""
+    if kind == "free" and len(I) == 1:
+        pytest.skip("needs a vector to give the batch size")
+    ho, so = orc.make_hashes(420, I, J, D)
+    fT = synth.gaussian(421, (D, sum(J) - len(J) + 1))
+    v = [synth.unit_vectors(422 + n, B, i) for n, i in enumerate(I)]
+    hg, sg, fg, vg = cuda(ho), cuda(so), cuda(fT), [cuda(x) for x in v]
+    f64, v64 = fT.astype(np.float64), [x.astype(np.float64) for x in v]
+    ra = rf = None
+    if kind == "both":
+        _, _, ra, rf = fcs.fcs_contract_both(ctx, fg, vg, I, J, hg, sg, free_mode=m, raw=True)
+    elif kind == "all":
+        _, ra = fcs.fcs_contract(ctx, fcs.FCS_CONTRACT_ALL, fg, vg, I, J, hg, sg, raw=True)
+    else:
+        med, rf = fcs.fcs_contract(ctx, fcs.FCS_CONTRACT_FREE, fg, vg, I, J, hg, sg, free_mode=m,
+                                   raw=True)
+    for b in range(B):
+        vb = [x[b] for x in v64]
+        if ra is not None:
+            ref = orc.contract_all(f64, vb, J, ho, so)
+            scale = np.linalg.norm(f64, axis=1)
+            assert np.all(np.abs(host(ra)[b] - ref) <= CONTRACT_RTOL * scale)
+        if rf is not None:
+            ref = orc.contract_free(f64, vb, m, J, ho, so)
+            err = np.linalg.norm(host(rf)[b] - ref, axis=1)
+            assert np.all(err <= CONTRACT_RTOL * np.linalg.norm(ref, axis=1))
