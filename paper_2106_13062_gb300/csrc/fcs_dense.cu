@@ -165,9 +165,9 @@ __global__ void __launch_bounds__(1024) dense_kernel(DenseArgs a) {
 // Accumulation is exact integer fixed point: shared-memory FP32 atomics are a
 // compare-and-swap loop (about 6x slower than a 32-bit integer atomic add), so
 // every entry x is rounded once to xi = rint(x / q) with a power-of-two step
-// q = 2^(E-25) per CTA, where 2^E bounds the magnitudes of a sample (the first
-// row of every warp), and the D signed copies of xi are added with int32
-// atomics.  Integer sums do not depend on the order of the adds.  Three cases
+// q = 2^(E-25) per CTA (down to 2^(E-27) for short last modes), where 2^E
+// bounds the magnitudes of a sample (the first row of every warp), and the D
+// signed copies of xi are added with int32 atomics.  Integer sums do not depend on the order of the adds.  Three cases
 // leave the fast path, each exactly:
 //  * outliers (|x| >= ~2^30 q, NaN, Inf) are added in FP32 straight into the
 //    output sketch with global atomics;
@@ -180,15 +180,18 @@ __global__ void __launch_bounds__(1024) dense_kernel(DenseArgs a) {
 //    q sqrt(n/12) for n rounded entries, exceeds 1e-7 of the CTA's
 //    ||x||_2 (data with a large dynamic range), the CTA re-reads its rows and
 //    adds the exact remainders x - q xi with FP32 shared atomics.
-// A CTA whose sample is all zeros or outside 2^-100..2^100 accumulates in FP32.
+// A CTA whose sample is all zeros or outside 2^-98..2^100 accumulates in FP32.
 // The bins are flushed to the output as FP32 (q xi_sum, one rounding).
 // Hash values outside [0, J_n) are skipped; a CTA that finds one in its
 // tables takes the checked (slower) scatter for every row.
 // NL = number of leading modes (N - 1) when known at compile time, -1 for the
 // general case (N - 1 <= kMaxN - 1, checked at run time).
-template <int NT, int NL>
+// FLAT: one row of CTAs over all tensors of a batch, each with an equal run of
+// the flat_rows rows of the batch, instead of blockIdx.y naming the tensor.
+template <int NT, int NL, bool FLAT>
 __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, int cpr,
-                                                        int64_t warps_used, int DC) {
+                                                        int64_t warps_used, int DC,
+                                                        int64_t flat_rows) {
   constexpr int NLMAX = NL >= 0 ? NL : kMaxN - 1;
   auto leading = [&](int n) { return n < NLMAX && (NL >= 0 || n < a.m.N - 1); };
   // this CTA handles sketches d0 .. d0 + nd - 1 (nd <= DC); d below is local
@@ -231,9 +234,9 @@ __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, i
   for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) ibins[e] = 0;
 
   const int lane = threadIdx.x & 31;
-  const int64_t gw = (blockIdx.x * int64_t(NT) + threadIdx.x) >> 5;
+  const int64_t gw = ((FLAT ? 0 : blockIdx.x * int64_t(NT)) + threadIdx.x) >> 5;
   const int c = int(gw % cpr);
-  const int64_t rstride = warps_used / cpr;
+  const uint32_t rstride = uint32_t(warps_used / cpr);
   const int64_t i0 = int64_t(c) * 256 + lane * 4;      // segment s starts at i0 + 128 s
   const bool act0 = i0 < a.L, act1 = i0 + 128 < a.L;
   // last-mode tables in shared memory, one 16-byte word per (sketch, chunk,
@@ -273,12 +276,12 @@ __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, i
   for (int k = threadIdx.x; k < nd * cpr * 32 * 8; k += NT)
     reinterpret_cast<uint16_t *>(ltab)[k] &= uint16_t(0x7fff);
 
-  const int b = blockIdx.y;
-  const float *Tb = a.T + b * a.tbs;
-  float *outb = a.out + b * a.obs;
+  // the tensor at hand, and the rows [rbeg, rend) of it that this CTA takes
+  uint32_t rbeg = 0, rend = uint32_t(a.rows);
+  const float *Tb = nullptr;
+  float *outb = nullptr;
   // rows < 2^31 and I_n < 2^31 here, so 32-bit division suffices
-  auto row_addr = [&](int64_t row, int *idx) {
-    uint32_t rr = uint32_t(row);
+  auto row_addr = [&](uint32_t rr, int *idx) {
     int64_t addr = 0;
 #pragma unroll
     for (int n = NLMAX - 1; n >= 0; --n) {
@@ -329,248 +332,288 @@ __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, i
               : make_float4(0.f, 0.f, 0.f, 0.f);
   };
   const bool working = gw < warps_used;
-  const int64_t row0 = gw / cpr;
+  const uint32_t wrow = uint32_t(gw / cpr);
 
-  // ---- scale from the sample: the first row of every warp
-  {
-    float m = 0.f;
-    if (working && row0 < a.rows) {
-      int idx[kMaxN];
-      float4 x0, x1;
-      load(row_addr(row0, idx), x0, x1);
-      const float v[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+  auto tensor_part = [&](int64_t b) {
+    Tb = a.T + b * a.tbs;
+    outb = a.out + b * a.obs;
+    const uint32_t row0 = rbeg + wrow;
+    // ---- scale from the sample: the first row of every warp
+    {
+      float m = 0.f;
+      if (working && row0 < rend) {
+        int idx[kMaxN];
+        float4 x0, x1;
+        load(row_addr(row0, idx), x0, x1);
+        const float v[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if (fabsf(v[e]) <= FLT_MAX) m = fmaxf(m, fabsf(v[e]));
+        for (int e = 0; e < 8; ++e)
+          if (fabsf(v[e]) <= FLT_MAX) m = fmaxf(m, fabsf(v[e]));
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0 && m > 0.f) atomicMax(&s_max, __float_as_uint(m));
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0 && m > 0.f) atomicMax(&s_max, __float_as_uint(m));
-  }
-  __syncthreads();
-  const bool tables_ok = s_bad == 0;
-  int E = 0;
-  const float smax = __uint_as_float(s_max);
-  frexpf(smax, &E);                        // smax < 2^E
-  const bool fx = smax > 0.f && E > -100 && E < 100;
-  const float q = fx ? ldexpf(1.f, E - 25) : 1.f;        // fixed-point step
-  const float inv_q = fx ? ldexpf(1.f, 25 - E) : 1.f;
-  const float carry = fx ? ldexpf(1.f, E + 7) : 0.f;     // 2^32 q
+    __syncthreads();
+    const bool tables_ok = s_bad == 0;
+    // Fixed-point step q = 2^(E - sh) for a sample maximum smax = frac 2^E: 25
+    // bits, and up to two more where that would take the second pass below for
+    // ordinary data (which counts the lanes past the end of a short last mode as
+    // rounded entries: pad of them to a real one; at smax = 3.7 deviations the
+    // tested ratio is 1e-15 pad / frac^2 against 1e-14) and the bins have room (m
+    // entries to a bin reach about 1.5 sqrt(m) smax / 3.7 in the middle of a
+    // sketch).  32 tensors of 100^3 at D = 5: 678 us with 25 bits always, 221 so;
+    // 1000 of 300 x 40 at D = 10 491 and 348; q is never coarser than with 25.
+    int E = 0;
+    const float smax = __uint_as_float(s_max);
+    const float frac = frexpf(smax, &E);
+    const float pad = float(cpr) * 256.f / float(a.L);
+    const float m_bin = float(rend - rbeg) * float(a.L) / (float(Jt) * float(FLAT ? 1 : gridDim.x));
+    const float fill = sqrtf(m_bin) * frac;
+    const int sh = 25 + int(pad > 3.5f * frac * frac && fill <= 21.f) +
+                   int(pad > 14.f * frac * frac && fill <= 10.f);
+    const bool fx = smax > 0.f && E > -98 && E < 100;
+    const float q = fx ? ldexpf(1.f, E - sh) : 1.f;
+    const float inv_q = fx ? ldexpf(1.f, sh - E) : 1.f;
+    const float carry = fx ? ldexpf(1.f, E - sh + 32) : 0.f;     // 2^32 q
 
-  // Fast scatter of one row into sketch d: eight int32 adds issued back to
-  // back, then one test of their old values (bit 31 of old + 2^30 is set iff
-  // |old| >= 2^30); only then are the adds checked for a wrap.  LNEG is the
-  // leading modes' sign, uniform across the warp.  The lane's table and bin
-  // pointers for sketch d are passed in (stepped once per sketch).
-  const uint4 *ltab_l = reinterpret_cast<const uint4 *>(ltab) + c * 32 + lane;
-  const uint32_t *lsg_l = lsg + c * 32 + lane;
-  const int lstep = cpr * 32;
-  auto scatter_fast = [&](auto lneg_c, int d, int base, const int *xi, const uint4 *tp,
-                          const uint32_t *sp, int32_t *bins_d) {
-    constexpr bool LNEG = decltype(lneg_c)::value;
-    const uint4 tw = *tp;
-    const uint32_t w[4] = {tw.x, tw.y, tw.z, tw.w};
-    const uint32_t sg = *sp;
-    int32_t *bb = bins_d + base;
-    int val[8], old[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const uint32_t off = (e & 1) ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xffffu);
-      const bool sneg = ((sg >> e) & 1u) != 0;
-      val[e] = (sneg != LNEG) ? -xi[e] : xi[e];
-      old[e] = atomicAdd(bb + off, val[e]);
-    }
-    // bit 31 of old + 2^30 is set iff |old| >= 2^30
-    int flag = 0;
-#pragma unroll
-    for (int e = 0; e < 8; e += 2)
-      flag |= int(unsigned(old[e]) + 0x40000000u) | int(unsigned(old[e + 1]) + 0x40000000u);
-    if (flag < 0) {                                    // rare: a large bin
-      float *od = outb + (d0 + d) * Jt + base;
+    // Fast scatter of one row into sketch d: eight int32 adds issued back to
+    // back, then one test of their old values (bit 31 of old + 2^30 is set iff
+    // |old| >= 2^30); only then are the adds checked for a wrap.  LNEG is the
+    // leading modes' sign, uniform across the warp.  The lane's table and bin
+    // pointers for sketch d are passed in (stepped once per sketch).
+    const uint4 *ltab_l = reinterpret_cast<const uint4 *>(ltab) + c * 32 + lane;
+    const uint32_t *lsg_l = lsg + c * 32 + lane;
+    const int lstep = cpr * 32;
+    auto scatter_fast = [&](auto lneg_c, int d, int base, const int *xi, const uint4 *tp,
+                            const uint32_t *sp, int32_t *bins_d) {
+      constexpr bool LNEG = decltype(lneg_c)::value;
+      const uint4 tw = *tp;
+      const uint32_t w[4] = {tw.x, tw.y, tw.z, tw.w};
+      const uint32_t sg = *sp;
+      int32_t *bb = bins_d + base;
+      int val[8], old[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const uint32_t off = (e & 1) ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xffffu);
-        const int nw = int(unsigned(old[e]) + unsigned(val[e]));
-        if (((old[e] ^ nw) & (val[e] ^ nw)) < 0)
-          atomicAdd(od + off, val[e] > 0 ? carry : -carry);
+        const bool sneg = ((sg >> e) & 1u) != 0;
+        val[e] = (sneg != LNEG) ? -xi[e] : xi[e];
+        old[e] = atomicAdd(bb + off, val[e]);
       }
-    }
-  };
+      // bit 31 of old + 2^30 is set iff |old| >= 2^30
+      int flag = 0;
+#pragma unroll
+      for (int e = 0; e < 8; e += 2)
+        flag |= int(unsigned(old[e]) + 0x40000000u) | int(unsigned(old[e + 1]) + 0x40000000u);
+      if (flag < 0) {                                    // rare: a large bin
+        float *od = outb + (d0 + d) * Jt + base;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const uint32_t off = (e & 1) ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xffffu);
+          const int nw = int(unsigned(old[e]) + unsigned(val[e]));
+          if (((old[e] ^ nw) & (val[e] ^ nw)) < 0)
+            atomicAdd(od + off, val[e] > 0 ? carry : -carry);
+        }
+      }
+    };
 
-  // mode 0: fixed point (+ outliers, carries); 1: FP32 remainders x - q xi
-  // of the fixed-point entries; 2: plain FP32 accumulation.
-  float sumsq = 0.f;
-  unsigned nfx = 0;
-  auto run_rows = [&](auto mode_c) {
-    constexpr int MODE = decltype(mode_c)::value;
-    int64_t row = row0;
-    int idx[kMaxN], nidx[kMaxN];
+    // mode 0: fixed point (+ outliers, carries); 1: FP32 remainders x - q xi
+    // of the fixed-point entries; 2: plain FP32 accumulation.
+    float sumsq = 0.f;
+    unsigned nfx = 0;
+    auto run_rows = [&](auto mode_c) {
+      constexpr int MODE = decltype(mode_c)::value;
+      uint32_t row = row0;
+      int idx[kMaxN], nidx[kMaxN];
 #pragma unroll
-    for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n] = 0;
-    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
-    if (working && row < a.rows) load(row_addr(row, nidx), n0, n1);
-    for (; working && row < a.rows; row += rstride) {
+      for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n] = 0;
+      float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+      if (working && row < rend) load(row_addr(row, nidx), n0, n1);
+      for (; working && row < rend; row += rstride) {
 #pragma unroll
-      for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n];
-      const float v[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
-      if (row + rstride < a.rows) load(next_row(idx, nidx), n0, n1);
-      int xi[8];
-      float rv[8];
-      // one sum of squares per row decides the fast path: below 2^60 every
-      // |u| < 2^30 and nothing is NaN or Inf
-      float srow = 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float u = v[e] * inv_q;
-        xi[e] = __float2int_rn(u);
-        srow = fmaf(u, u, srow);
-      }
-      const bool fast_row =
-          MODE == 0 && tables_ok && __all_sync(0xffffffffu, srow < 1.152921504606846976e18f);
-      unsigned fastm = 0xffu;      // bit e: entry e goes through the integer path
-      if (MODE == 0) {
-        sumsq += srow;             // in units of q^2
-        nfx += 8u;
-      }
-      if (!fast_row) {
-        fastm = 0u;
+        for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n];
+        const float v[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
+        if (row + rstride < rend) load(next_row(idx, nidx), n0, n1);
+        int xi[8];
+        float rv[8];
+        // one sum of squares per row decides the fast path: below 2^60 every
+        // |u| < 2^30 and nothing is NaN or Inf
+        float srow = 0.f;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const float u = v[e] * inv_q;
-          const bool fast = fabsf(u) < 1073741760.f;     // 2^30 - 2^6; false for NaN
-          if (!fast) xi[e] = 0;
-          fastm |= unsigned(fast) << e;
-          rv[e] = MODE == 1 ? (fast ? fmaf(-q, __int2float_rn(xi[e]), v[e]) : 0.f) : v[e];
+          xi[e] = __float2int_rn(u);
+          srow = fmaf(u, u, srow);
         }
-      }
-      if (fast_row) {
-        const int32_t *tabn[kMaxN];
+        const bool fast_row =
+            MODE == 0 && tables_ok && __all_sync(0xffffffffu, srow < 1.152921504606846976e18f);
+        unsigned fastm = 0xffu;      // bit e: entry e goes through the integer path
+        if (MODE == 0) {
+          sumsq += srow;             // in units of q^2
+          nfx += 8u;
+        }
+        if (!fast_row) {
+          fastm = 0u;
 #pragma unroll
-        for (int n = 0; n < NLMAX; ++n)
-          if (leading(n)) tabn[n] = tab + int(a.coff[n] + idx[n]);
-        const uint4 *tp = ltab_l;
-        const uint32_t *sp = lsg_l;
-        int32_t *bins_d = ibins;
+          for (int e = 0; e < 8; ++e) {
+            const float u = v[e] * inv_q;
+            const bool fast = fabsf(u) < 1073741760.f;     // 2^30 - 2^6; false for NaN
+            if (!fast) xi[e] = 0;
+            fastm |= unsigned(fast) << e;
+            rv[e] = MODE == 1 ? (fast ? fmaf(-q, __int2float_rn(xi[e]), v[e]) : 0.f) : v[e];
+          }
+        }
+        if (fast_row) {
+          const int32_t *tabn[kMaxN];
+#pragma unroll
+          for (int n = 0; n < NLMAX; ++n)
+            if (leading(n)) tabn[n] = tab + int(a.coff[n] + idx[n]);
+          const uint4 *tp = ltab_l;
+          const uint32_t *sp = lsg_l;
+          int32_t *bins_d = ibins;
+#pragma unroll 1
+          for (int d = 0; d < nd; ++d) {
+            int base = 0, neg = 0;
+#pragma unroll
+            for (int n = 0; n < NLMAX; ++n) {
+              if (leading(n)) {
+                const int32_t t = *tabn[n];
+                tabn[n] += totL;
+                base += t >> 1;
+                neg ^= t & 1;
+              }
+            }
+            if (neg)
+              scatter_fast(std::true_type(), d, base, xi, tp, sp, bins_d);
+            else
+              scatter_fast(std::false_type(), d, base, xi, tp, sp, bins_d);
+            tp += lstep;
+            sp += lstep;
+            bins_d += Jt;
+          }
+          continue;
+        }
+        // checked scatter (bad hash values, outliers, FP32 modes): the tables
+        // are re-read from global memory and every index is checked
 #pragma unroll 1
         for (int d = 0; d < nd; ++d) {
           int base = 0, neg = 0;
+          bool row_ok = true;
 #pragma unroll
           for (int n = 0; n < NLMAX; ++n) {
             if (leading(n)) {
-              const int32_t t = *tabn[n];
-              tabn[n] += totL;
+              const int32_t t = tab[d * totL + int(a.coff[n] + idx[n])];
               base += t >> 1;
               neg ^= t & 1;
+              row_ok = row_ok && unsigned(t >> 1) < unsigned(a.m.J[n]);
             }
           }
-          if (neg)
-            scatter_fast(std::true_type(), d, base, xi, tp, sp, bins_d);
-          else
-            scatter_fast(std::false_type(), d, base, xi, tp, sp, bins_d);
-          tp += lstep;
-          sp += lstep;
-          bins_d += Jt;
-        }
-        continue;
-      }
-      // checked scatter (bad hash values, outliers, FP32 modes): the tables
-      // are re-read from global memory and every index is checked
-#pragma unroll 1
-      for (int d = 0; d < nd; ++d) {
-        int base = 0, neg = 0;
-        bool row_ok = true;
+          if (!row_ok) continue;
+          int32_t *bi = ibins + d * Jt + base;
+          float *bf = fbins + d * Jt + base;
+          float *od = outb + (d0 + d) * Jt + base;
+          const uint32_t JL = uint32_t(a.m.J[N - 1]);
 #pragma unroll
-        for (int n = 0; n < NLMAX; ++n) {
-          if (leading(n)) {
-            const int32_t t = tab[d * totL + int(a.coff[n] + idx[n])];
-            base += t >> 1;
-            neg ^= t & 1;
-            row_ok = row_ok && unsigned(t >> 1) < unsigned(a.m.J[n]);
-          }
-        }
-        if (!row_ok) continue;
-        int32_t *bi = ibins + d * Jt + base;
-        float *bf = fbins + d * Jt + base;
-        float *od = outb + (d0 + d) * Jt + base;
-        const uint32_t JL = uint32_t(a.m.J[N - 1]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          if (!((e < 4) ? act0 : act1)) continue;
-          const int64_t il = i0 + (e >> 2) * 128 + (e & 3);
-          const int32_t t = packed_entry(a, d0 + d, int(a.m.off[N - 1] + il));
-          const uint32_t off = uint32_t(t >> 1);
-          if (off >= JL) continue;
-          const bool sneg = ((t & 1) != 0) != (neg != 0);
-          if (MODE == 0) {
-            if ((fastm >> e) & 1u) {
-              const int val = sneg ? -xi[e] : xi[e];
-              const int old = atomicAdd(bi + off, val);
-              const int nw = int(unsigned(old) + unsigned(val));
-              if (((old ^ nw) & (val ^ nw)) < 0) atomicAdd(od + off, val > 0 ? carry : -carry);
-            } else {
-              atomicAdd(od + off, sneg ? -v[e] : v[e]);   // outlier, exact FP32
+          for (int e = 0; e < 8; ++e) {
+            if (!((e < 4) ? act0 : act1)) continue;
+            const int64_t il = i0 + (e >> 2) * 128 + (e & 3);
+            const int32_t t = packed_entry(a, d0 + d, int(a.m.off[N - 1] + il));
+            const uint32_t off = uint32_t(t >> 1);
+            if (off >= JL) continue;
+            const bool sneg = ((t & 1) != 0) != (neg != 0);
+            if (MODE == 0) {
+              if ((fastm >> e) & 1u) {
+                const int val = sneg ? -xi[e] : xi[e];
+                const int old = atomicAdd(bi + off, val);
+                const int nw = int(unsigned(old) + unsigned(val));
+                if (((old ^ nw) & (val ^ nw)) < 0) atomicAdd(od + off, val > 0 ? carry : -carry);
+              } else {
+                atomicAdd(od + off, sneg ? -v[e] : v[e]);   // outlier, exact FP32
+              }
+            } else if (MODE == 2 || ((fastm >> e) & 1u)) {
+              atomicAdd(bf + off, sneg ? -rv[e] : rv[e]);
             }
-          } else if (MODE == 2 || ((fastm >> e) & 1u)) {
-            atomicAdd(bf + off, sneg ? -rv[e] : rv[e]);
           }
         }
       }
-    }
-  };
-  // Add the CTA's bins (value(e) for local bin e) to the output: 16-byte
-  // vector reductions over the aligned middle, scalar atomics at the ends.
-  auto flush = [&](auto value) {
-    float *dst = outb + d0 * Jt;
-    const int64_t n = nd * Jt;
-    int64_t head = int64_t((16 - (reinterpret_cast<uintptr_t>(dst) & 15)) & 15) / 4;
-    if (head > n) head = n;
-    const int64_t body = head + ((n - head) & ~int64_t(3));
-    for (int64_t e = threadIdx.x; e < head; e += NT) {
-      const float x = value(e);
-      if (x != 0.f) atomicAdd(dst + e, x);
-    }
-    for (int64_t e = head + 4 * int64_t(threadIdx.x); e < body; e += 4 * int64_t(NT)) {
-      const float x0 = value(e), x1 = value(e + 1), x2 = value(e + 2), x3 = value(e + 3);
-      if (x0 != 0.f || x1 != 0.f || x2 != 0.f || x3 != 0.f)
-        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e), "f"(x0),
-                     "f"(x1), "f"(x2), "f"(x3)
-                     : "memory");
-    }
-    for (int64_t e = body + threadIdx.x; e < n; e += NT) {
-      const float x = value(e);
-      if (x != 0.f) atomicAdd(dst + e, x);
-    }
-  };
-  auto flush_float = [&]() { flush([&](int64_t e) { return fbins[e]; }); };
+    };
+    // Add the CTA's bins (value(e) for local bin e) to the output: 16-byte
+    // vector reductions over the aligned middle, scalar atomics at the ends.
+    auto flush = [&](auto value) {
+      float *dst = outb + d0 * Jt;
+      const int64_t n = nd * Jt;
+      int64_t head = int64_t((16 - (reinterpret_cast<uintptr_t>(dst) & 15)) & 15) / 4;
+      if (head > n) head = n;
+      const int64_t body = head + ((n - head) & ~int64_t(3));
+      for (int64_t e = threadIdx.x; e < head; e += NT) {
+        const float x = value(e);
+        if (x != 0.f) atomicAdd(dst + e, x);
+      }
+      for (int64_t e = head + 4 * int64_t(threadIdx.x); e < body; e += 4 * int64_t(NT)) {
+        const float x0 = value(e), x1 = value(e + 1), x2 = value(e + 2), x3 = value(e + 3);
+        if (x0 != 0.f || x1 != 0.f || x2 != 0.f || x3 != 0.f)
+          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e), "f"(x0),
+                       "f"(x1), "f"(x2), "f"(x3)
+                       : "memory");
+      }
+      for (int64_t e = body + threadIdx.x; e < n; e += NT) {
+        const float x = value(e);
+        if (x != 0.f) atomicAdd(dst + e, x);
+      }
+    };
+    auto flush_float = [&]() { flush([&](int64_t e) { return fbins[e]; }); };
 
-  if (!fx) {                          // this CTA accumulates in FP32
-    run_rows(std::integral_constant<int, 2>());
+    if (!fx) {                          // this CTA accumulates in FP32
+      run_rows(std::integral_constant<int, 2>());
+      __syncthreads();
+      flush_float();
+      return;
+    }
+    run_rows(std::integral_constant<int, 0>());
+    // CTA totals for the rounding-error test
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      sumsq += __shfl_xor_sync(0xffffffffu, sumsq, o);
+      nfx += __shfl_xor_sync(0xffffffffu, nfx, o);
+    }
+    if (lane == 0) {
+      atomicAdd(&s_sumsq, sumsq);
+      atomicAdd(&s_nfx, (unsigned long long)nfx);
+    }
+    __syncthreads();
+    flush([&](int64_t e) { return __int2float_rn(ibins[e]) * q; });
+    // expected squared rounding error n q^2 / 12 against (1e-7 ||x||)^2, in
+    // units of q^2 (the test is uniform across the CTA)
+    if (!(float(s_nfx) * (1.f / 12.f) > 1e-14f * s_sumsq)) return;
+    __syncthreads();
+    for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) fbins[e] = 0.f;
+    __syncthreads();
+    run_rows(std::integral_constant<int, 1>());
     __syncthreads();
     flush_float();
-    return;
+  };
+
+  if constexpr (!FLAT) {
+    tensor_part(blockIdx.y);
+  } else {
+    int64_t f = flat_rows * blockIdx.x / gridDim.x;
+    for (;;) {
+      const int64_t f1 = flat_rows * (blockIdx.x + 1) / gridDim.x, b = f / a.rows;
+      rbeg = uint32_t(f - b * a.rows);
+      rend = uint32_t(min(a.rows, rbeg + (f1 - f)));
+      f += rend - rbeg;
+      tensor_part(b);
+      if (f >= f1) break;
+      __syncthreads();
+      for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) ibins[e] = 0;
+      if (threadIdx.x == 0) {
+        s_max = 0u;
+        s_sumsq = 0.f;
+        s_nfx = 0ull;
+      }
+      __syncthreads();
+    }
   }
-  run_rows(std::integral_constant<int, 0>());
-  // CTA totals for the rounding-error test
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    sumsq += __shfl_xor_sync(0xffffffffu, sumsq, o);
-    nfx += __shfl_xor_sync(0xffffffffu, nfx, o);
-  }
-  if (lane == 0) {
-    atomicAdd(&s_sumsq, sumsq);
-    atomicAdd(&s_nfx, (unsigned long long)nfx);
-  }
-  __syncthreads();
-  flush([&](int64_t e) { return __int2float_rn(ibins[e]) * q; });
-  // expected squared rounding error n q^2 / 12 against (1e-7 ||x||)^2, in
-  // units of q^2 (the test is uniform across the CTA)
-  if (!(float(s_nfx) * (1.f / 12.f) > 1e-14f * s_sumsq)) return;
-  __syncthreads();
-  for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) fbins[e] = 0.f;
-  __syncthreads();
-  run_rows(std::integral_constant<int, 1>());
-  __syncthreads();
-  flush_float();
 }
 
 }  // namespace
@@ -709,7 +752,7 @@ extern "C" int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
   const size_t smem_rows = rows_smem(DC);
   if (vec && a.m.J[N - 1] <= 32767 && smem_rows <= 200 * 1024 && a.rows < (int64_t(1) << 31)) {
     const int cpr = cpr_rows;
-    auto launch_rows = [&](auto kern, int nt) -> int {
+    auto launch_rows = [&](auto kern, auto kern_flat, int nt) -> int {
       if (smem_rows > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              int(smem_rows));
@@ -733,16 +776,42 @@ extern "C" int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
         per_item = (int64_t(cpr) * 32 + nt - 1) / nt;
         used = cpr;
       }
+      // Batches whose tensors' CTAs leave a quarter of the SMs idle or make
+      // several waves: one wave of CTAs with equal runs of rows of the whole
+      // batch, each of which builds its tables once and adds its bins out after
+      // every tensor.  512 x 512 at D = 10 (us, a block per tensor / so): 100
+      // tensors 162 / 122, 160 317 / 182, 256 323 / 283, 1000 1126 / 1054; with 128
+      // CTAs for 152 SMs (32 tensors) it was no faster, 52 / 52 (at D = 1 15 / 18).
+      const int64_t want = std::max<int64_t>(1, int64_t(ctx->sm_count) * per_sm / ngroups);
+      const int64_t ctas = per_item * nbatch;
+      const int nw = nt / 32;
+      const bool uneven = ctas > want || ctas * 4 <= want * 3;
+      if (nbatch > 1 && uneven && cpr <= nw && (nw % cpr) * 8 <= nw &&
+          a.rows * nbatch >= 4 * (nw / cpr) * want) {
+        if (smem_rows > 48 * 1024) {
+          cudaError_t e = cudaFuncSetAttribute(
+              kern_flat, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_rows));
+          if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(dense_rows)");
+        }
+        kern_flat<<<dim3(unsigned(want), 1u, unsigned(ngroups)), nt, smem_rows, ctx->stream>>>(
+            a, int(totL), cpr, nw / cpr * cpr, DC, a.rows * nbatch);
+        return check_cuda(ctx, cudaGetLastError(), "dense_rows_kernel");
+      }
       kern<<<dim3(unsigned(per_item), unsigned(nbatch), unsigned(ngroups)), nt, smem_rows,
-             ctx->stream>>>(a, int(totL), cpr, used, DC);
+             ctx->stream>>>(a, int(totL), cpr, used, DC, 0);
       return check_cuda(ctx, cudaGetLastError(), "dense_rows_kernel");
     };
     switch (N - 1) {
-      case 0: return launch_rows(dense_rows_kernel<768, 0>, 768);
-      case 1: return launch_rows(dense_rows_kernel<768, 1>, 768);
-      case 2: return launch_rows(dense_rows_kernel<768, 2>, 768);
-      case 3: return launch_rows(dense_rows_kernel<768, 3>, 768);
-      default: return launch_rows(dense_rows_kernel<768, -1>, 768);
+      case 0:
+        return launch_rows(dense_rows_kernel<768, 0, false>, dense_rows_kernel<768, 0, true>, 768);
+      case 1:
+        return launch_rows(dense_rows_kernel<768, 1, false>, dense_rows_kernel<768, 1, true>, 768);
+      case 2:
+        return launch_rows(dense_rows_kernel<768, 2, false>, dense_rows_kernel<768, 2, true>, 768);
+      case 3:
+        return launch_rows(dense_rows_kernel<768, 3, false>, dense_rows_kernel<768, 3, true>, 768);
+      default:
+        return launch_rows(dense_rows_kernel<768, -1, false>, dense_rows_kernel<768, -1, true>, 768);
     }
   }
   if (vec)

@@ -76,6 +76,28 @@ def test_dense_small_tensor_nan_and_bad_hash(fcs, ctx, orc):
     assert np.linalg.norm(got[fin] - ref[fin]) <= 1e-5 * np.linalg.norm(ref[fin])
 
 
+@pytest.mark.parametrize("shape,J,D,nb", [
+    ((20, 16, 260), [90, 80, 300], 2, 33), ((12, 260), [50, 400], 3, 640), ((400,), [300], 1, 20000),
+    ((4, 2, 3, 2, 2, 96), [9, 5, 7, 3, 4, 50], 2, 160), ((16, 16, 64), [3000, 3000, 3000], 10, 100),
+])
+@pytest.mark.parametrize("kind", ["normal", "spike", "nan"])
+def test_dense_batch_rows(fcs, ctx, orc, shape, J, D, nb, kind):
+    """Batches whose rows are shared out evenly over the CTAs, so that a CTA
+    takes parts of several tensors: a large value or a NaN stays in its own."""
+    T = synth.gaussian(411, (nb,) + shape)
+    if kind != "normal":
+        T.reshape(nb, -1)[nb // 2, 0] = 3e9 if kind == "spike" else np.nan
+    ho, so = orc.make_hashes(412, list(shape), J, D)
+    got = host(fcs.fcs_sketch_dense(ctx, cuda(T), J, cuda(ho), cuda(so), batched=True))
+    pick = sorted({0, 1, nb // 2 - 1, nb // 2, nb // 2 + 1, nb - 1})
+    ref = _dense_ref(orc, T[pick], J, ho, so)
+    fin = np.isfinite(ref)
+    assert np.array_equal(np.isfinite(got[pick]), fin)
+    assert np.isfinite(got).sum() == got.size - (~fin).sum()
+    for g, r, f in zip(got[pick], ref, fin):
+        assert np.linalg.norm(g[f] - r[f]) <= 1e-5 * np.linalg.norm(r[f])
+
+
 @pytest.mark.parametrize("B,C,D,Jt", [(1, 1, 1, 1), (5, 3, 16, 31), (256, 10, 5, 178), (6, 130, 2, 33),
                                       (700, 9, 3, 1000), (2000, 200, 2, 40)])
 def test_inner_products(fcs, ctx, B, C, D, Jt):
