@@ -317,8 +317,8 @@ class DenseWorkload:
         return self.D
 
     def launches_per_step(self):
-        # hashes, zero + dense, spectrum, fused contraction, 2 medians
-        return 1 + 2 + 1 + 1 + 2
+        # hashes, zero + dense, spectrum, fused contraction, medians
+        return 1 + 2 + 1 + 1 + 1
 
     def bytes(self):
         """Dense kernel: the tensor read once, tables read once, sketches
@@ -743,8 +743,8 @@ class BatchWorkload:
                                             ["fcs_batch.cu", "fcs_batch_kernels.cuh",
                                              "fcs_batch_k0.cu", "fcs_batch_k1.cu",
                                              "fcs_batch_k2.cu", "fcs_batch_k3.cu",
-                                             "fcs_batch_k4.cu", "fcs_cp_run.cuh", "fcs_fft.cuh",
-                                             "fcs_internal.cuh"]),
+                                             "fcs_batch_k4.cu", "fcs_cp_run.cuh", "fcs_pair.cuh",
+                                             "fcs_fft.cuh", "fcs_internal.cuh"]),
                 "peak_source": f"derived: {props.multi_processor_count} SMs x 128 FP32 lanes "
                                f"x 2 flop/FMA x {sm_mhz:.0f} MHz",
                 "avg_launch_ms": t, "grain": self.grain,

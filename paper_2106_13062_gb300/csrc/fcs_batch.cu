@@ -10,10 +10,9 @@
 // transpose every problem's factor columns in one batched launch, run one
 // kernel per FFT size -- so it can be captured into a CUDA graph and
 // replayed.  Device side: each size class runs with the block size and
-// engine of the single-problem kernel for that size (cp_run / cp13_run of
+// engine of the single-problem kernel for that size (cp_run / cp_pair_run of
 // fcs_cp_run.cuh), one CTA per item: count sketch into a compact shared
-// buffer, block real FFT, mode product in registers, rank sum in shared
-// memory, the item's partial spectrum into the problem's accumulator, and
+// buffer, real FFT, mode product and rank sum on the SM, the item's partial spectrum into the problem's accumulator, and
 // the item that completes sketch (p, d) (ticket counter) runs that sketch's
 // inverse FFT.  The class launches form a chain of programmatic dependent
 // launches, so a class starts while the previous one drains.  No CTA ever

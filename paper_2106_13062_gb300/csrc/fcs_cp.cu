@@ -8,14 +8,13 @@
 // the spectrum accumulator and, for fcs_sketch_cp_seeded, writes the hash
 // tables of a seed (the same entries as fcs_make_hashes).  The sketch kernel
 // is its programmatic dependent: placed while prep runs, it waits for the
-// prep grid at its first instruction.  (2) The fused sketch kernel: CTA (g, d) owns
-// sketch d and a contiguous group of ranks and runs cp_run (P <= 8192) or
-// cp13_run (P = 16384) of fcs_cp_run.cuh: count sketch, block real FFT, mode
+// prep grid before it reads what that writes.  (2) The fused sketch kernel: each
+// CTA works on one sketch d and some of the ranks and runs cp_run (P <= 4096) or
+// cp_pair_run (P = 8192 .. 32768) of fcs_cp_run.cuh: count sketch, real FFT, mode
 // product and rank sum in the frequency domain (linearity moves the paper's
 // sum of inverse transforms inside one inverse transform), partial spectrum
 // into a global accumulator, and the one inverse FFT by the CTA that
-// completes sketch d.  Longer transforms go to the two-pass route of
-// fcs_big.cu.
+// completes sketch d.  Longer transforms go to the routes of fcs_big.cu.
 #include <algorithm>
 #include <cstdarg>
 #include <mutex>
