@@ -858,7 +858,8 @@ class BatchPlan:
     def __init__(self, ctx: Context, problems, grain: int = 0, classes=None):
         """classes: None (autotuned or default shapes) or a list of
         (fft_len, thread_mult, items_per_cta[, engine]) per FFT-length class;
-        engine 0 = slot FFT, 1 = row-pair (default: 1 for P = 8192 and 16384, else 0)."""
+        engine 0 = slot FFT, 1 = warp-DIT (P = 8192) or row-pair (P = 16384), the
+        default at these two."""
         self.ctx = ctx
         self._arr = _problem_array(problems)
         h = C.c_void_p()

@@ -10,8 +10,8 @@
 // transpose every problem's factor columns in one batched launch, run one
 // kernel per FFT size -- so it can be captured into a CUDA graph and
 // replayed.  Device side: each size class runs with the block size and
-// engine of the single-problem kernel for that size (cp_run / cp_pair_run of
-// fcs_cp_run.cuh), one CTA per item: count sketch into a compact shared
+// engine of the single-problem kernel for that size (cp_run, cp12_run or
+// cp_pair_run of fcs_cp_run.cuh), one CTA per item: count sketch into a compact shared
 // buffer, real FFT, mode product and rank sum on the SM, the item's partial spectrum into the problem's accumulator, and
 // the item that completes sketch (p, d) (ticket counter) runs that sketch's
 // inverse FFT.  The class launches form a chain of programmatic dependent
@@ -102,12 +102,12 @@ __global__ void __launch_bounds__(256) batch_transpose_kernel(const TransposeTas
   }
 }
 
-// Engine of a class without a tuned or explicit shape: the row-pair engine
-// where it exists (P = 8192 .. 32768), the slot FFT below.
+// Engine of a class without a tuned or explicit shape: the warp-DIT engine at
+// P = 8192, the row-pair engine beyond, the slot FFT below.
 int default_engine(int L) { return L >= 12 ? 1 : 0; }
 
 // Class kernel for log2 M = L with engine eng, at thread multiplier ntm (slot
-// FFT only; the row-pair engine has one thread count) running ipc items
+// FFT only; the other engines have one thread count) running ipc items
 // per CTA.
 ClassKernel class_kernel(int L, int eng, int ntm, int ipc, int64_t Imax, int sb) {
   if (L >= 13) return class_kernel_13(L, ipc, sb);
@@ -159,7 +159,7 @@ int check_problem(fcs_ctx *ctx, int k, const fcs_cp_problem &q, HostProb *hp) {
   hp->longp = log2p > kMaxLog2P + 1 || (log2p == kMaxLog2P + 1 && jmax > kPair32MaxJ);
   hp->L = log2p - 1;
   hp->sb = int((jmax + 3) / 4 * 4);
-  hp->tall = hp->L == 12 ? hp->sb > pair_full_sb<8>() : hp->L == 13 ? hp->sb > pair_full_sb<16>() : 0;
+  hp->tall = hp->L == 13 && hp->sb > pair_full_sb<16>();
   hp->R = q.R;
   hp->utlen = ut;
   hp->Imax = imax;
@@ -791,7 +791,7 @@ extern "C" int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem 
     const ClassCfg keep = *c;
     ClassCfg bestc = keep;
     // shapes (engine, threads): slot FFT at 1 or 2 x the threads; for
-    // P = 8192 also the row-pair engine, the only one beyond
+    // P = 8192 also the warp-DIT engine, beyond only the row-pair engine
     std::vector<std::pair<int, int>> shapes;
     if (c->L >= 13) {
       shapes = {{1, 1}};

@@ -9,13 +9,13 @@
 namespace fcs {
 
 // Tunable shape of one FFT-size class (log2 M = L): the engine (for P = 8192
-// the slot FFT or the row-pair engine; beyond, always the row-pair engine, the
+// the slot FFT or the warp-DIT engine; beyond, always the row-pair engine, the
 // other sizes the slot FFT), the slot FFT's thread multiplier ntm (1 or 2:
 // M/16 or M/8 threads, at least a warp) and items run one after another per
 // CTA (ipc: 1, 2 or 4).
 struct ClassCfg {
   int L, ntm, ipc;
-  int eng = 0;               // P = 8192: 0 = slot FFT, 1 = row-pair engine
+  int eng = 0;               // P = 8192: 0 = slot FFT, 1 = warp-DIT engine
 };
 
 // One launch of a batch: the items [first, first + count) of one FFT size.

@@ -27,7 +27,7 @@ struct BatchProb {
   int pad_;
 };
 
-// cp_run / cp_pair_run's accessors over a problem descriptor (fcs_cp_run.cuh).
+// The accessors of fcs_cp_run.cuh over a problem descriptor.
 struct BatchView {
   const BatchProb &P;
   int sb;
@@ -123,6 +123,35 @@ __global__ void __launch_bounds__(NT) batch_class_kernel(const BatchProb *__rest
     const int first = blockIdx.x * ipc, last = min(count, first + ipc);
     for (int it = first; it < last; ++it) {
       if (it > first) __syncthreads();       // shared memory of the previous item
+      one(it);
+    }
+  } else {
+    one(blockIdx.x);
+  }
+  pdl_wait_previous();
+}
+
+// The same for P = 8192 on the warp-DIT engine (256 threads, two CTAs per SM;
+// ra <= 32 RMAX).
+template <int CPT, int RMAX, bool MULTI>
+__global__ void __launch_bounds__(wdit::kNT, 2) batch_class12w_kernel(
+    const BatchProb *__restrict__ probs, const int4 *__restrict__ items,
+    const float2 *__restrict__ tw, int count, int ipc) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int is_last;
+  pdl_launch_dependents();
+  auto one = [&](int it) {
+    const int4 w = items[it];
+    const BatchProb &P = probs[w.x];
+    const int64_t r0 = int64_t(w.z) * P.rpi;
+    const int64_t r1 = min(P.R, r0 + P.rpi);
+    const BatchView view{P, P.sb};
+    cp12_run<CPT, RMAX>(view, w.y, r0, r1, unsigned(P.groups), smem_raw, tw, &is_last);
+  };
+  if constexpr (MULTI) {
+    const int first = blockIdx.x * ipc, last = min(count, first + ipc);
+    for (int it = first; it < last; ++it) {
+      if (it > first) __syncthreads();
       one(it);
     }
   } else {

@@ -9,8 +9,8 @@
 // tables of a seed (the same entries as fcs_make_hashes).  The sketch kernel
 // is its programmatic dependent: placed while prep runs, it waits for the
 // prep grid before it reads what that writes.  (2) The fused sketch kernel: each
-// CTA works on one sketch d and some of the ranks and runs cp_run (P <= 4096) or
-// cp_pair_run (P = 8192 .. 32768) of fcs_cp_run.cuh: count sketch, real FFT, mode
+// CTA works on one sketch d and some of the ranks and runs cp_run (P <= 4096),
+// cp12_run (P = 8192) or cp_pair_run (P = 16384, 32768) of fcs_cp_run.cuh: count sketch, real FFT, mode
 // product and rank sum in the frequency domain (linearity moves the paper's
 // sum of inverse transforms inside one inverse transform), partial spectrum
 // into a global accumulator, and the one inverse FFT by the CTA that
@@ -58,14 +58,14 @@ struct TransposeArgs {
 // of the prep launch, so their CTAs are placed while prep runs.  Every one of
 // them waits for the prep grid to complete (and its writes to be visible:
 // transposed factors, cleared accumulator and tickets, hash tables) before
-// anything that touches those: cp_kernel first of all, cp_pair_kernel once
+// anything that touches those: cp_kernel and cp12_kernel first of all, cp_pair_kernel once
 // its tables and scatter buffer are set up.  Launched the ordinary way the
 // wait returns at once.
 __device__ __forceinline__ void wait_for_prep() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// cp_run / cp_pair_run's accessors over CpArgs (fcs_cp_run.cuh).
+// The accessors of fcs_cp_run.cuh over CpArgs.
 struct CpView {
   const CpArgs &a;
   int sb;
@@ -131,6 +131,19 @@ __global__ void __launch_bounds__(NT) cp_kernel(CpArgs a, const float2 *__restri
   const int64_t r1 = min(a.R, r0 + a.ranks_per_cta);
   const CpView view{a, a.sb};
   cp_run<LOG2M, NT, CPT>(view, blockIdx.y, r0, r1, gridDim.x, smem_raw, tw, &is_last);
+}
+
+// The same for P = 8192 on the warp-DIT engine (256 threads, two CTAs per
+// SM).  RMAX = number of 32-entry blocks per scatter-buffer row.
+template <int CPT, int RMAX>
+__global__ void __launch_bounds__(wdit::kNT, 2) cp12_kernel(CpArgs a, const float2 *__restrict__ tw) {
+  wait_for_prep();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int is_last;
+  const int64_t r0 = blockIdx.x * a.ranks_per_cta;
+  const int64_t r1 = min(a.R, r0 + a.ranks_per_cta);
+  const CpView view{a, a.sb};
+  cp12_run<CPT, RMAX>(view, blockIdx.y, r0, r1, gridDim.x, smem_raw, tw, &is_last);
 }
 
 // The same for P = 1024 NR on the row-pair engine.  A one-dimensional grid:
@@ -253,9 +266,39 @@ cudaError_t launch_pair(CpArgs &a, int sm_count, const float2 *tw, cudaStream_t 
                            args);
 }
 
+// Warp-DIT kernel for the given prefetch depth and scatter-buffer height.
+template <int CPT>
+const void *cp12_pick(int ra) {
+  if (ra <= 128) return reinterpret_cast<const void *>(cp12_kernel<CPT, 4>);
+  if (ra <= 256) return reinterpret_cast<const void *>(cp12_kernel<CPT, 8>);
+  return reinterpret_cast<const void *>(cp12_kernel<CPT, 16>);
+}
+cudaError_t launch_cp12(CpArgs &a, int64_t groups, int64_t Imax, const float2 *tw,
+                        cudaStream_t st) {
+  const int ra = (a.sb + 15) >> 4;
+  const size_t smem = Cp12Smem::bytes(ra);
+  const int cpt = int((Imax + wdit::kNT - 1) / wdit::kNT);
+  const void *kern = cpt <= 1 ? cp12_pick<1>(ra) : cpt <= 2 ? cp12_pick<2>(ra) : cp12_pick<4>(ra);
+  const cudaError_t e = allow_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  void *args[] = {&a, &tw};
+  return launch_after_prep(st, kern, dim3(unsigned(groups), unsigned(a.D)), dim3(wdit::kNT), smem,
+                           args);
+}
+
+// Split a.R into groups of equal ranks for about `slots` CTAs in all; returns
+// the number of groups per sketch.
+int64_t even_groups(CpArgs &a, int64_t slots) {
+  const int64_t g = std::min(a.R, std::max<int64_t>(1, (slots + a.D - 1) / a.D));
+  a.ranks_per_cta = (a.R + g - 1) / g;
+  return (a.R + a.ranks_per_cta - 1) / a.ranks_per_cta;
+}
+
 template <int LOG2M>
 int launch_cp(fcs_ctx *ctx, CpArgs &a, int64_t groups, int64_t Imax) {
-  if constexpr (LOG2M >= 12) {
+  if constexpr (LOG2M == 12) {
+    return check_cuda(ctx, launch_cp12(a, groups, Imax, ctx->twiddle, ctx->stream), "cp12_kernel");
+  } else if constexpr (LOG2M > 12) {
     return check_cuda(ctx,
                       launch_pair<1 << (LOG2M - 9), CpView>(a, ctx->sm_count, ctx->twiddle,
                                                             ctx->stream),
@@ -350,12 +393,9 @@ int sketch_cp_impl(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t *ho
   a.h = h;
   a.s = s;
   a.out = out;
-  // rank groups of the slot FFT: about one CTA per SM over all sketches
-  int64_t groups = (int64_t(ctx->sm_count) + D - 1) / D;
-  if (groups < 1) groups = 1;
-  if (groups > R) groups = R;
-  a.ranks_per_cta = (R + groups - 1) / groups;
-  groups = (R + a.ranks_per_cta - 1) / a.ranks_per_cta;
+  // rank groups of the engines below P = 16384: about one CTA per SM over all
+  // sketches (two for P = 8192, whose engine fits two CTAs per SM)
+  const int64_t groups = even_groups(a, int64_t(ctx->sm_count) * (log2m == 12 ? 2 : 1));
 
   a.sb = int((Jmax + 3) / 4 * 4);
   void *ws = nullptr;
@@ -545,7 +585,12 @@ int noalloc_setup(int dev, cudaStream_t st, NoAllocDevice **out, char *err, size
 template <int LOG2M>
 int noalloc_launch_cp(CpArgs &a, int64_t groups, int64_t Imax, int sm_count, const float2 *tw,
                       cudaStream_t st, char *err, size_t n) {
-  if constexpr (LOG2M >= 12) {
+  if constexpr (LOG2M == 12) {
+    const cudaError_t e = launch_cp12(a, groups, Imax, tw, st);
+    if (e != cudaSuccess)
+      return noalloc_fail(err, n, FCS_ECUDA, "cp12_kernel: %s", cudaGetErrorString(e));
+    return FCS_OK;
+  } else if constexpr (LOG2M > 12) {
     const cudaError_t e = launch_pair<1 << (LOG2M - 9), CpView>(a, sm_count, tw, st);
     if (e != cudaSuccess)
       return noalloc_fail(err, n, FCS_ECUDA, "cp_pair_kernel: %s", cudaGetErrorString(e));
@@ -637,11 +682,7 @@ extern "C" int fcs_sketch_cp_noalloc(void *stream, int N, const int64_t *host_I,
   a.s = s;
   a.out = out;
   a.sb = int((Jmax + 3) / 4 * 4);
-  int64_t groups = (int64_t(sd->sm_count) + D - 1) / D;
-  if (groups < 1) groups = 1;
-  if (groups > R) groups = R;
-  a.ranks_per_cta = (R + groups - 1) / groups;
-  groups = (R + a.ranks_per_cta - 1) / a.ranks_per_cta;
+  const int64_t groups = even_groups(a, int64_t(sd->sm_count) * (log2m == 12 ? 2 : 1));
   a.G = reinterpret_cast<float2 *>(sd->scratch);
   a.counter = reinterpret_cast<unsigned *>(sd->scratch + gbytes);
   float *UT = reinterpret_cast<float *>(sd->scratch + gbytes + cbytes);

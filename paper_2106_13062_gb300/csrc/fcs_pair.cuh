@@ -1,5 +1,5 @@
 // fcs_pair.cuh -- the forward real FFT of the CP route for P = 1024 NR,
-// NR = 8, 16 or 32 (M = 512 NR complex points), on packed FP32 arithmetic.
+// NR = 16 or 32 (M = 512 NR complex points), on packed FP32 arithmetic.
 //
 // The transform is a decimation in time over NR rows of 512 points,
 //   Z[k + 512 q1] = sum_w W_NR^(w q1) W_M^(w k) Y_w[k],  Y_w = FFT_512(z[NR m + w]).
@@ -31,8 +31,8 @@
 // A rank's running mode product and the rank sum (64 words each per thread,
 // 128 at NR = 32) live in tensor memory: they are touched once per transform,
 // and without them a thread's 32 spectrum values and the temporaries fit 128
-// registers, so two 256-thread CTAs (four of 128 threads at NR = 8) share an
-// SM and one's barriers hide behind the other.
+// registers, so two 256-thread CTAs share an SM at NR = 16 and one's barriers
+// hide behind the other.
 #pragma once
 
 #include "fcs_fft.cuh"
@@ -133,8 +133,9 @@ struct Geo {
   static constexpr int LNR = log2_const(NR);
   static constexpr int M = 512 * NR;
   static constexpr int LM = 9 + LNR;                  // log2 M
-  static constexpr int NT = NR == 8 ? 128 : 256;      // threads per CTA
-  static constexpr int CTAS = NR == 8 ? 4 : NR == 16 ? 2 : 1;   // CTAs per SM
+  static_assert(NR == 16 || NR == 32, "P = 16384 or 32768");
+  static constexpr int NT = 256;                      // threads per CTA
+  static constexpr int CTAS = NR == 16 ? 2 : 1;       // CTAs per SM
   static constexpr int WARPS = NT / 32;
   static constexpr int RPW = NR / 2 / WARPS;          // row pairs per warp
   static constexpr int NCP = 256 / NT;                // column pairs per thread
