@@ -543,6 +543,7 @@ int fcs_rtpm(fcs_ctx *ctx, int N, int64_t I, const int32_t *host_J, int D, const
  * G = *_{n != m} F_n F_n^T (Cholesky) and column normalisation.
  * host_F[n]: device [R][I_n], the transposed factor matrices (row r = column
  * r of U_n): starting values in, unit-norm factors out; lambda [R] out.
+ * Modes may share a factor buffer; each then sees the other's updates.
  */
 int fcs_als(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t *host_J, int D,
             const float *fcsT, const int32_t *h, const int8_t *s, int64_t ldh, int R,

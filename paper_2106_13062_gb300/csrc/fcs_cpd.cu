@@ -85,6 +85,7 @@ struct AlsArgs {
   float *gram;           // [N][R][R]: F_n F_n^T
   float *lambda;         // [R]
   int in_smem;           // the solution fits shared memory
+  unsigned shared;       // bit n: F_n shares memory with F_m (n != m)
 };
 
 // g = V V^T for V [R][I]: one warp per pair of rows, two pairs at a time.
@@ -142,12 +143,6 @@ __global__ void __launch_bounds__(kUpdNT) als_update_kernel(AlsArgs a) {
   __shared__ float G[kMaxRank][kMaxRank + 1];
   __shared__ float sums[kUpdNT / RM][RM];
   __shared__ float nrm[RM], inv[RM];
-  // x / g from inv = 1 / g, with the remainder added back (a division's slow
-  // path would cost the solve its registers)
-  auto quotient = [](float x, float g, float inv) {
-    const float q = x * inv;
-    return fmaf(fmaf(-q, g, x), inv, q);
-  };
   const int R = a.R, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   for (int p = tid; p < RM * RM; p += kUpdNT) {
     const int r = p / RM, q = p % RM;
@@ -250,6 +245,8 @@ __global__ void __launch_bounds__(kUpdNT) als_update_kernel(AlsArgs a) {
   }
   __syncthreads();
   gram_matrix(X, Im, R, a.gram + a.m * R * R);
+  for (int n = 0; n < a.N; ++n)
+    if (a.shared >> n & 1u) gram_matrix(a.F[n], a.I[n], R, a.gram + n * R * R);
 }
 
 // Turns the spectrum cache on for the duration of a call and restores it.
@@ -402,6 +399,11 @@ extern "C" int fcs_als(fcs_ctx *ctx, int N, const int64_t *host_I, const int32_t
       a.m = mm;
       const size_t xb = sizeof(float) * size_t(R) * size_t(host_I[mm]);
       a.in_smem = xb <= 40 * 1024;
+      a.shared = 0;
+      for (int n = 0; n < N; ++n)
+        if (n != mm && host_F[n] < host_F[mm] + R * host_I[mm] &&
+            host_F[mm] < host_F[n] + R * host_I[n])
+          a.shared |= 1u << n;
       const size_t xsm = a.in_smem ? xb : 0;
       if (R <= 8)
         als_update_kernel<8><<<1, kUpdNT, xsm, ctx->stream>>>(a);
