@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "fcs_div.cuh"
 #include "fcs_internal.cuh"
 
 namespace fcs {
@@ -131,7 +132,7 @@ __global__ void __launch_bounds__(1024) als_gram_kernel(AlsArgs a) {
 // One CTA: G = *_{n != m} F_n F_n^T from the Gram matrices, Cholesky G = L
 // L^T, then for every column i of M^T the solve G x = M^T[:, i]; row norms give
 // lambda and the normalised rows the new F_m, whose Gram matrix replaces the
-// old one.  Latency-bound (400 x 10: 50 us with the Gram products of whole
+// old one (as do those of modes whose factors lie in the same memory).  Latency-bound (400 x 10: 50 us with the Gram products of whole
 // rows by one thread each, the factorisation by one thread and the solve's
 // vector in local memory; now 20 us): a warp factors, lane i holding row i, and
 // RM >= R lanes solve eight columns at a time, one element of each per lane (the
