@@ -186,15 +186,12 @@ __global__ void __launch_bounds__(1024) dense_kernel(DenseArgs a) {
 // tables takes the checked (slower) scatter for every row.
 // NL = number of leading modes (N - 1) when known at compile time, -1 for the
 // general case (N - 1 <= kMaxN - 1, checked at run time).
-// FLAT: one row of CTAs over all tensors of a batch, each with an equal run of
-// the flat_rows rows of the batch, instead of blockIdx.y naming the tensor.
 // FINE: a last mode that leaves a sixth of its chunks' lanes without entries or
 // more; its fixed-point step may have more bits (a variant of its own: in the
 // others the same lines cost 0.5 to 1.8 % of a 53 us launch).
-template <int NT, int NL, bool FLAT, bool FINE>
+template <int NT, int NL, bool FINE>
 __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, int cpr,
-                                                        int64_t warps_used, int DC,
-                                                        int64_t flat_rows) {
+                                                        int64_t warps_used, int DC) {
   constexpr int NLMAX = NL >= 0 ? NL : kMaxN - 1;
   auto leading = [&](int n) { return n < NLMAX && (NL >= 0 || n < a.m.N - 1); };
   // this CTA handles sketches d0 .. d0 + nd - 1 (nd <= DC); d below is local
@@ -237,7 +234,7 @@ __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, i
   for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) ibins[e] = 0;
 
   const int lane = threadIdx.x & 31;
-  const int64_t gw = ((FLAT ? 0 : blockIdx.x * int64_t(NT)) + threadIdx.x) >> 5;
+  const int64_t gw = (blockIdx.x * int64_t(NT) + threadIdx.x) >> 5;
   const int c = int(gw % cpr);
   const uint32_t rstride = uint32_t(warps_used / cpr);
   const int64_t i0 = int64_t(c) * 256 + lane * 4;      // segment s starts at i0 + 128 s
@@ -279,10 +276,10 @@ __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, i
   for (int k = threadIdx.x; k < nd * cpr * 32 * 8; k += NT)
     reinterpret_cast<uint16_t *>(ltab)[k] &= uint16_t(0x7fff);
 
-  // the tensor at hand, and the rows [rbeg, rend) of it that this CTA takes
-  uint32_t rbeg = 0, rend = uint32_t(a.rows);
-  const float *Tb = nullptr;
-  float *outb = nullptr;
+  const int b = blockIdx.y;
+  const float *Tb = a.T + b * a.tbs;
+  float *outb = a.out + b * a.obs;
+  const uint32_t rows = uint32_t(a.rows);
   // rows < 2^31 and I_n < 2^31 here, so 32-bit division suffices
   auto row_addr = [&](uint32_t rr, int *idx) {
     int64_t addr = 0;
@@ -335,292 +332,265 @@ __global__ void __launch_bounds__(NT) dense_rows_kernel(DenseArgs a, int totL, i
               : make_float4(0.f, 0.f, 0.f, 0.f);
   };
   const bool working = gw < warps_used;
-  const uint32_t wrow = uint32_t(gw / cpr);
+  const uint32_t row0 = uint32_t(gw / cpr);
 
-  auto tensor_part = [&](int64_t b) {
-    Tb = a.T + b * a.tbs;
-    outb = a.out + b * a.obs;
-    const uint32_t row0 = rbeg + wrow;
-    // ---- scale from the sample: the first row of every warp
-    {
-      float m = 0.f;
-      if (working && row0 < rend) {
-        int idx[kMaxN];
-        float4 x0, x1;
-        load(row_addr(row0, idx), x0, x1);
-        const float v[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+  // ---- scale from the sample: the first row of every warp
+  {
+    float m = 0.f;
+    if (working && row0 < rows) {
+      int idx[kMaxN];
+      float4 x0, x1;
+      load(row_addr(row0, idx), x0, x1);
+      const float v[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (fabsf(v[e]) <= FLT_MAX) m = fmaxf(m, fabsf(v[e]));
-      }
+      for (int e = 0; e < 8; ++e)
+        if (fabsf(v[e]) <= FLT_MAX) m = fmaxf(m, fabsf(v[e]));
+    }
 #pragma unroll
-      for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0 && m > 0.f) atomicMax(&s_max, __float_as_uint(m));
-    }
-    __syncthreads();
-    const bool tables_ok = s_bad == 0;
-    // Fixed-point step q = 2^(E - sh) for a sample maximum smax = frac 2^E: 25
-    // bits, and up to two more where that would take the second pass below for
-    // ordinary data (which counts the lanes past the end of a short last mode as
-    // rounded entries: pad of them to a real one; at smax = 3.7 deviations the
-    // tested ratio is 1e-15 pad / frac^2 against 1e-14) and the bins have room (m
-    // entries to a bin reach about 1.5 sqrt(m) smax / 3.7 in the middle of a
-    // sketch).  32 tensors of 100^3 at D = 5: 678 us with 25 bits always, 221 so;
-    // 1000 of 300 x 40 at D = 10 491 and 348; q is never coarser than with 25.
-    int E = 0;
-    const float smax = __uint_as_float(s_max);
-    const float frac = frexpf(smax, &E);
-    int sh = 25;
-    if constexpr (FINE) {
-      const float pad = float(cpr) * 256.f / float(a.L);
-      const float m_bin =
-          float(rend - rbeg) * float(a.L) / (float(Jt) * float(FLAT ? 1 : gridDim.x));
-      const float fill = sqrtf(m_bin) * frac;
-      sh += int(pad > 3.5f * frac * frac && fill <= 21.f) +
-            int(pad > 14.f * frac * frac && fill <= 10.f);
-    }
-    const bool fx = smax > 0.f && E > -98 && E < 100;
-    const float q = fx ? ldexpf(1.f, E - sh) : 1.f;
-    const float inv_q = fx ? ldexpf(1.f, sh - E) : 1.f;
-    const float carry = fx ? ldexpf(1.f, E - sh + 32) : 0.f;     // 2^32 q
+    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0 && m > 0.f) atomicMax(&s_max, __float_as_uint(m));
+  }
+  __syncthreads();
+  const bool tables_ok = s_bad == 0;
+  // Fixed-point step q = 2^(E - sh) for a sample maximum smax = frac 2^E: 25
+  // bits, and up to two more where that would take the second pass below for
+  // ordinary data (which counts the lanes past the end of a short last mode as
+  // rounded entries: pad of them to a real one; at smax = 3.7 deviations the
+  // tested ratio is 1e-15 pad / frac^2 against 1e-14) and the bins have room (m
+  // entries to a bin reach about 1.5 sqrt(m) smax / 3.7 in the middle of a
+  // sketch).  32 tensors of 100^3 at D = 5: 678 us with 25 bits always, 221 so;
+  // 1000 of 300 x 40 at D = 10 491 and 348; q is never coarser than with 25.
+  int E = 0;
+  const float smax = __uint_as_float(s_max);
+  const float frac = frexpf(smax, &E);
+  int sh = 25;
+  if constexpr (FINE) {
+    const float pad = float(cpr) * 256.f / float(a.L);
+    const float m_bin =
+        float(rows) * float(a.L) / (float(Jt) * float(gridDim.x));
+    const float fill = sqrtf(m_bin) * frac;
+    sh += int(pad > 3.5f * frac * frac && fill <= 21.f) +
+          int(pad > 14.f * frac * frac && fill <= 10.f);
+  }
+  const bool fx = smax > 0.f && E > -98 && E < 100;
+  const float q = fx ? ldexpf(1.f, E - sh) : 1.f;
+  const float inv_q = fx ? ldexpf(1.f, sh - E) : 1.f;
+  const float carry = fx ? ldexpf(1.f, E - sh + 32) : 0.f;     // 2^32 q
 
-    // Fast scatter of one row into sketch d: eight int32 adds issued back to
-    // back, then one test of their old values (bit 31 of old + 2^30 is set iff
-    // |old| >= 2^30); only then are the adds checked for a wrap.  LNEG is the
-    // leading modes' sign, uniform across the warp.  The lane's table and bin
-    // pointers for sketch d are passed in (stepped once per sketch).
-    const uint4 *ltab_l = reinterpret_cast<const uint4 *>(ltab) + c * 32 + lane;
-    const uint32_t *lsg_l = lsg + c * 32 + lane;
-    const int lstep = cpr * 32;
-    auto scatter_fast = [&](auto lneg_c, int d, int base, const int *xi, const uint4 *tp,
-                            const uint32_t *sp, int32_t *bins_d) {
-      constexpr bool LNEG = decltype(lneg_c)::value;
-      const uint4 tw = *tp;
-      const uint32_t w[4] = {tw.x, tw.y, tw.z, tw.w};
-      const uint32_t sg = *sp;
-      int32_t *bb = bins_d + base;
-      int val[8], old[8];
+  // Fast scatter of one row into sketch d: eight int32 adds issued back to
+  // back, then one test of their old values (bit 31 of old + 2^30 is set iff
+  // |old| >= 2^30); only then are the adds checked for a wrap.  LNEG is the
+  // leading modes' sign, uniform across the warp.  The lane's table and bin
+  // pointers for sketch d are passed in (stepped once per sketch).
+  const uint4 *ltab_l = reinterpret_cast<const uint4 *>(ltab) + c * 32 + lane;
+  const uint32_t *lsg_l = lsg + c * 32 + lane;
+  const int lstep = cpr * 32;
+  auto scatter_fast = [&](auto lneg_c, int d, int base, const int *xi, const uint4 *tp,
+                          const uint32_t *sp, int32_t *bins_d) {
+    constexpr bool LNEG = decltype(lneg_c)::value;
+    const uint4 tw = *tp;
+    const uint32_t w[4] = {tw.x, tw.y, tw.z, tw.w};
+    const uint32_t sg = *sp;
+    int32_t *bb = bins_d + base;
+    int val[8], old[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const uint32_t off = (e & 1) ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xffffu);
+      const bool sneg = ((sg >> e) & 1u) != 0;
+      val[e] = (sneg != LNEG) ? -xi[e] : xi[e];
+      old[e] = atomicAdd(bb + off, val[e]);
+    }
+    // bit 31 of old + 2^30 is set iff |old| >= 2^30
+    int flag = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e += 2)
+      flag |= int(unsigned(old[e]) + 0x40000000u) | int(unsigned(old[e + 1]) + 0x40000000u);
+    if (flag < 0) {                                    // rare: a large bin
+      float *od = outb + (d0 + d) * Jt + base;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const uint32_t off = (e & 1) ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xffffu);
-        const bool sneg = ((sg >> e) & 1u) != 0;
-        val[e] = (sneg != LNEG) ? -xi[e] : xi[e];
-        old[e] = atomicAdd(bb + off, val[e]);
+        const int nw = int(unsigned(old[e]) + unsigned(val[e]));
+        if (((old[e] ^ nw) & (val[e] ^ nw)) < 0)
+          atomicAdd(od + off, val[e] > 0 ? carry : -carry);
       }
-      // bit 31 of old + 2^30 is set iff |old| >= 2^30
-      int flag = 0;
-#pragma unroll
-      for (int e = 0; e < 8; e += 2)
-        flag |= int(unsigned(old[e]) + 0x40000000u) | int(unsigned(old[e + 1]) + 0x40000000u);
-      if (flag < 0) {                                    // rare: a large bin
-        float *od = outb + (d0 + d) * Jt + base;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const uint32_t off = (e & 1) ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xffffu);
-          const int nw = int(unsigned(old[e]) + unsigned(val[e]));
-          if (((old[e] ^ nw) & (val[e] ^ nw)) < 0)
-            atomicAdd(od + off, val[e] > 0 ? carry : -carry);
-        }
-      }
-    };
+    }
+  };
 
-    // mode 0: fixed point (+ outliers, carries); 1: FP32 remainders x - q xi
-    // of the fixed-point entries; 2: plain FP32 accumulation.
-    float sumsq = 0.f;
-    unsigned nfx = 0;
-    auto run_rows = [&](auto mode_c) {
-      constexpr int MODE = decltype(mode_c)::value;
-      uint32_t row = row0;
-      int idx[kMaxN], nidx[kMaxN];
+  // mode 0: fixed point (+ outliers, carries); 1: FP32 remainders x - q xi
+  // of the fixed-point entries; 2: plain FP32 accumulation.
+  float sumsq = 0.f;
+  unsigned nfx = 0;
+  auto run_rows = [&](auto mode_c) {
+    constexpr int MODE = decltype(mode_c)::value;
+    uint32_t row = row0;
+    int idx[kMaxN], nidx[kMaxN];
 #pragma unroll
-      for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n] = 0;
-      float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
-      if (working && row < rend) load(row_addr(row, nidx), n0, n1);
-      for (; working && row < rend; row += rstride) {
+    for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n] = 0;
+    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+    if (working && row < rows) load(row_addr(row, nidx), n0, n1);
+    for (; working && row < rows; row += rstride) {
 #pragma unroll
-        for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n];
-        const float v[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
-        if (row + rstride < rend) load(next_row(idx, nidx), n0, n1);
-        int xi[8];
-        float rv[8];
-        // one sum of squares per row decides the fast path: below 2^60 every
-        // |u| < 2^30 and nothing is NaN or Inf
-        float srow = 0.f;
+      for (int n = 0; n < kMaxN; ++n) idx[n] = nidx[n];
+      const float v[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
+      if (row + rstride < rows) load(next_row(idx, nidx), n0, n1);
+      int xi[8];
+      float rv[8];
+      // one sum of squares per row decides the fast path: below 2^60 every
+      // |u| < 2^30 and nothing is NaN or Inf
+      float srow = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float u = v[e] * inv_q;
+        xi[e] = __float2int_rn(u);
+        srow = fmaf(u, u, srow);
+      }
+      const bool fast_row =
+          MODE == 0 && tables_ok && __all_sync(0xffffffffu, srow < 1.152921504606846976e18f);
+      unsigned fastm = 0xffu;      // bit e: entry e goes through the integer path
+      if (MODE == 0) {
+        sumsq += srow;             // in units of q^2
+        nfx += 8u;
+      }
+      if (!fast_row) {
+        fastm = 0u;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const float u = v[e] * inv_q;
-          xi[e] = __float2int_rn(u);
-          srow = fmaf(u, u, srow);
+          const bool fast = fabsf(u) < 1073741760.f;     // 2^30 - 2^6; false for NaN
+          if (!fast) xi[e] = 0;
+          fastm |= unsigned(fast) << e;
+          rv[e] = MODE == 1 ? (fast ? fmaf(-q, __int2float_rn(xi[e]), v[e]) : 0.f) : v[e];
         }
-        const bool fast_row =
-            MODE == 0 && tables_ok && __all_sync(0xffffffffu, srow < 1.152921504606846976e18f);
-        unsigned fastm = 0xffu;      // bit e: entry e goes through the integer path
-        if (MODE == 0) {
-          sumsq += srow;             // in units of q^2
-          nfx += 8u;
-        }
-        if (!fast_row) {
-          fastm = 0u;
+      }
+      if (fast_row) {
+        const int32_t *tabn[kMaxN];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float u = v[e] * inv_q;
-            const bool fast = fabsf(u) < 1073741760.f;     // 2^30 - 2^6; false for NaN
-            if (!fast) xi[e] = 0;
-            fastm |= unsigned(fast) << e;
-            rv[e] = MODE == 1 ? (fast ? fmaf(-q, __int2float_rn(xi[e]), v[e]) : 0.f) : v[e];
-          }
-        }
-        if (fast_row) {
-          const int32_t *tabn[kMaxN];
-#pragma unroll
-          for (int n = 0; n < NLMAX; ++n)
-            if (leading(n)) tabn[n] = tab + int(a.coff[n] + idx[n]);
-          const uint4 *tp = ltab_l;
-          const uint32_t *sp = lsg_l;
-          int32_t *bins_d = ibins;
-#pragma unroll 1
-          for (int d = 0; d < nd; ++d) {
-            int base = 0, neg = 0;
-#pragma unroll
-            for (int n = 0; n < NLMAX; ++n) {
-              if (leading(n)) {
-                const int32_t t = *tabn[n];
-                tabn[n] += totL;
-                base += t >> 1;
-                neg ^= t & 1;
-              }
-            }
-            if (neg)
-              scatter_fast(std::true_type(), d, base, xi, tp, sp, bins_d);
-            else
-              scatter_fast(std::false_type(), d, base, xi, tp, sp, bins_d);
-            tp += lstep;
-            sp += lstep;
-            bins_d += Jt;
-          }
-          continue;
-        }
-        // checked scatter (bad hash values, outliers, FP32 modes): the tables
-        // are re-read from global memory and every index is checked
+        for (int n = 0; n < NLMAX; ++n)
+          if (leading(n)) tabn[n] = tab + int(a.coff[n] + idx[n]);
+        const uint4 *tp = ltab_l;
+        const uint32_t *sp = lsg_l;
+        int32_t *bins_d = ibins;
 #pragma unroll 1
         for (int d = 0; d < nd; ++d) {
           int base = 0, neg = 0;
-          bool row_ok = true;
 #pragma unroll
           for (int n = 0; n < NLMAX; ++n) {
             if (leading(n)) {
-              const int32_t t = tab[d * totL + int(a.coff[n] + idx[n])];
+              const int32_t t = *tabn[n];
+              tabn[n] += totL;
               base += t >> 1;
               neg ^= t & 1;
-              row_ok = row_ok && unsigned(t >> 1) < unsigned(a.m.J[n]);
             }
           }
-          if (!row_ok) continue;
-          int32_t *bi = ibins + d * Jt + base;
-          float *bf = fbins + d * Jt + base;
-          float *od = outb + (d0 + d) * Jt + base;
-          const uint32_t JL = uint32_t(a.m.J[N - 1]);
+          if (neg)
+            scatter_fast(std::true_type(), d, base, xi, tp, sp, bins_d);
+          else
+            scatter_fast(std::false_type(), d, base, xi, tp, sp, bins_d);
+          tp += lstep;
+          sp += lstep;
+          bins_d += Jt;
+        }
+        continue;
+      }
+      // checked scatter (bad hash values, outliers, FP32 modes): the tables
+      // are re-read from global memory and every index is checked
+#pragma unroll 1
+      for (int d = 0; d < nd; ++d) {
+        int base = 0, neg = 0;
+        bool row_ok = true;
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            if (!((e < 4) ? act0 : act1)) continue;
-            const int64_t il = i0 + (e >> 2) * 128 + (e & 3);
-            const int32_t t = packed_entry(a, d0 + d, int(a.m.off[N - 1] + il));
-            const uint32_t off = uint32_t(t >> 1);
-            if (off >= JL) continue;
-            const bool sneg = ((t & 1) != 0) != (neg != 0);
-            if (MODE == 0) {
-              if ((fastm >> e) & 1u) {
-                const int val = sneg ? -xi[e] : xi[e];
-                const int old = atomicAdd(bi + off, val);
-                const int nw = int(unsigned(old) + unsigned(val));
-                if (((old ^ nw) & (val ^ nw)) < 0) atomicAdd(od + off, val > 0 ? carry : -carry);
-              } else {
-                atomicAdd(od + off, sneg ? -v[e] : v[e]);   // outlier, exact FP32
-              }
-            } else if (MODE == 2 || ((fastm >> e) & 1u)) {
-              atomicAdd(bf + off, sneg ? -rv[e] : rv[e]);
+        for (int n = 0; n < NLMAX; ++n) {
+          if (leading(n)) {
+            const int32_t t = tab[d * totL + int(a.coff[n] + idx[n])];
+            base += t >> 1;
+            neg ^= t & 1;
+            row_ok = row_ok && unsigned(t >> 1) < unsigned(a.m.J[n]);
+          }
+        }
+        if (!row_ok) continue;
+        int32_t *bi = ibins + d * Jt + base;
+        float *bf = fbins + d * Jt + base;
+        float *od = outb + (d0 + d) * Jt + base;
+        const uint32_t JL = uint32_t(a.m.J[N - 1]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          if (!((e < 4) ? act0 : act1)) continue;
+          const int64_t il = i0 + (e >> 2) * 128 + (e & 3);
+          const int32_t t = packed_entry(a, d0 + d, int(a.m.off[N - 1] + il));
+          const uint32_t off = uint32_t(t >> 1);
+          if (off >= JL) continue;
+          const bool sneg = ((t & 1) != 0) != (neg != 0);
+          if (MODE == 0) {
+            if ((fastm >> e) & 1u) {
+              const int val = sneg ? -xi[e] : xi[e];
+              const int old = atomicAdd(bi + off, val);
+              const int nw = int(unsigned(old) + unsigned(val));
+              if (((old ^ nw) & (val ^ nw)) < 0) atomicAdd(od + off, val > 0 ? carry : -carry);
+            } else {
+              atomicAdd(od + off, sneg ? -v[e] : v[e]);   // outlier, exact FP32
             }
+          } else if (MODE == 2 || ((fastm >> e) & 1u)) {
+            atomicAdd(bf + off, sneg ? -rv[e] : rv[e]);
           }
         }
       }
-    };
-    // Add the CTA's bins (value(e) for local bin e) to the output: 16-byte
-    // vector reductions over the aligned middle, scalar atomics at the ends.
-    auto flush = [&](auto value) {
-      float *dst = outb + d0 * Jt;
-      const int64_t n = nd * Jt;
-      int64_t head = int64_t((16 - (reinterpret_cast<uintptr_t>(dst) & 15)) & 15) / 4;
-      if (head > n) head = n;
-      const int64_t body = head + ((n - head) & ~int64_t(3));
-      for (int64_t e = threadIdx.x; e < head; e += NT) {
-        const float x = value(e);
-        if (x != 0.f) atomicAdd(dst + e, x);
-      }
-      for (int64_t e = head + 4 * int64_t(threadIdx.x); e < body; e += 4 * int64_t(NT)) {
-        const float x0 = value(e), x1 = value(e + 1), x2 = value(e + 2), x3 = value(e + 3);
-        if (x0 != 0.f || x1 != 0.f || x2 != 0.f || x3 != 0.f)
-          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e), "f"(x0),
-                       "f"(x1), "f"(x2), "f"(x3)
-                       : "memory");
-      }
-      for (int64_t e = body + threadIdx.x; e < n; e += NT) {
-        const float x = value(e);
-        if (x != 0.f) atomicAdd(dst + e, x);
-      }
-    };
-    auto flush_float = [&]() { flush([&](int64_t e) { return fbins[e]; }); };
+    }
+  };
+  // Add the CTA's bins (value(e) for local bin e) to the output: 16-byte
+  // vector reductions over the aligned middle, scalar atomics at the ends.
+  auto flush = [&](auto value) {
+    float *dst = outb + d0 * Jt;
+    const int64_t n = nd * Jt;
+    int64_t head = int64_t((16 - (reinterpret_cast<uintptr_t>(dst) & 15)) & 15) / 4;
+    if (head > n) head = n;
+    const int64_t body = head + ((n - head) & ~int64_t(3));
+    for (int64_t e = threadIdx.x; e < head; e += NT) {
+      const float x = value(e);
+      if (x != 0.f) atomicAdd(dst + e, x);
+    }
+    for (int64_t e = head + 4 * int64_t(threadIdx.x); e < body; e += 4 * int64_t(NT)) {
+      const float x0 = value(e), x1 = value(e + 1), x2 = value(e + 2), x3 = value(e + 3);
+      if (x0 != 0.f || x1 != 0.f || x2 != 0.f || x3 != 0.f)
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e), "f"(x0),
+                     "f"(x1), "f"(x2), "f"(x3)
+                     : "memory");
+    }
+    for (int64_t e = body + threadIdx.x; e < n; e += NT) {
+      const float x = value(e);
+      if (x != 0.f) atomicAdd(dst + e, x);
+    }
+  };
+  auto flush_float = [&]() { flush([&](int64_t e) { return fbins[e]; }); };
 
-    if (!fx) {                          // this CTA accumulates in FP32
-      run_rows(std::integral_constant<int, 2>());
-      __syncthreads();
-      flush_float();
-      return;
-    }
-    run_rows(std::integral_constant<int, 0>());
-    // CTA totals for the rounding-error test
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      sumsq += __shfl_xor_sync(0xffffffffu, sumsq, o);
-      nfx += __shfl_xor_sync(0xffffffffu, nfx, o);
-    }
-    if (lane == 0) {
-      atomicAdd(&s_sumsq, sumsq);
-      atomicAdd(&s_nfx, (unsigned long long)nfx);
-    }
-    __syncthreads();
-    flush([&](int64_t e) { return __int2float_rn(ibins[e]) * q; });
-    // expected squared rounding error n q^2 / 12 against (1e-7 ||x||)^2, in
-    // units of q^2 (the test is uniform across the CTA)
-    if (!(float(s_nfx) * (1.f / 12.f) > 1e-14f * s_sumsq)) return;
-    __syncthreads();
-    for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) fbins[e] = 0.f;
-    __syncthreads();
-    run_rows(std::integral_constant<int, 1>());
+  if (!fx) {                          // this CTA accumulates in FP32
+    run_rows(std::integral_constant<int, 2>());
     __syncthreads();
     flush_float();
-  };
-
-  if constexpr (!FLAT) {
-    tensor_part(blockIdx.y);
-  } else {
-    int64_t f = flat_rows * blockIdx.x / gridDim.x;
-    for (;;) {
-      const int64_t f1 = flat_rows * (blockIdx.x + 1) / gridDim.x, b = f / a.rows;
-      rbeg = uint32_t(f - b * a.rows);
-      rend = uint32_t(min(a.rows, rbeg + (f1 - f)));
-      f += rend - rbeg;
-      tensor_part(b);
-      if (f >= f1) break;
-      __syncthreads();
-      for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) ibins[e] = 0;
-      if (threadIdx.x == 0) {
-        s_max = 0u;
-        s_sumsq = 0.f;
-        s_nfx = 0ull;
-      }
-      __syncthreads();
-    }
+    return;
   }
+  run_rows(std::integral_constant<int, 0>());
+  // CTA totals for the rounding-error test
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    sumsq += __shfl_xor_sync(0xffffffffu, sumsq, o);
+    nfx += __shfl_xor_sync(0xffffffffu, nfx, o);
+  }
+  if (lane == 0) {
+    atomicAdd(&s_sumsq, sumsq);
+    atomicAdd(&s_nfx, (unsigned long long)nfx);
+  }
+  __syncthreads();
+  flush([&](int64_t e) { return __int2float_rn(ibins[e]) * q; });
+  // expected squared rounding error n q^2 / 12 against (1e-7 ||x||)^2, in
+  // units of q^2 (the test is uniform across the CTA)
+  if (!(float(s_nfx) * (1.f / 12.f) > 1e-14f * s_sumsq)) return;
+  __syncthreads();
+  for (int64_t e = threadIdx.x; e < nd * Jt; e += NT) fbins[e] = 0.f;
+  __syncthreads();
+  run_rows(std::integral_constant<int, 1>());
+  __syncthreads();
+  flush_float();
 }
 
 }  // namespace
@@ -759,7 +729,7 @@ extern "C" int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
   const size_t smem_rows = rows_smem(DC);
   if (vec && a.m.J[N - 1] <= 32767 && smem_rows <= 200 * 1024 && a.rows < (int64_t(1) << 31)) {
     const int cpr = cpr_rows;
-    auto launch_rows = [&](auto kern, auto kern_flat, int nt) -> int {
+    auto launch_rows = [&](auto kern, int nt) -> int {
       if (smem_rows > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              int(smem_rows));
@@ -783,38 +753,15 @@ extern "C" int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
         per_item = (int64_t(cpr) * 32 + nt - 1) / nt;
         used = cpr;
       }
-      // Batches whose tensors' CTAs leave a quarter of the SMs idle or make
-      // several waves: one wave of CTAs with equal runs of rows of the whole
-      // batch, each of which builds its tables once and adds its bins out after
-      // every tensor.  512 x 512 at D = 10 (us, a block per tensor / so): 100
-      // tensors 162 / 122, 160 317 / 182, 256 323 / 283, 1000 1126 / 1054; with 128
-      // CTAs for 152 SMs (32 tensors) it was no faster, 52 / 52 (at D = 1 15 / 18).
-      const int64_t want = std::max<int64_t>(1, int64_t(ctx->sm_count) * per_sm / ngroups);
-      const int64_t ctas = per_item * nbatch;
-      const int nw = nt / 32;
-      const bool uneven = ctas > want || ctas * 4 <= want * 3;
-      if (nbatch > 1 && uneven && cpr <= nw && (nw % cpr) * 8 <= nw &&
-          a.rows * nbatch >= 4 * (nw / cpr) * want) {
-        if (smem_rows > 48 * 1024) {
-          cudaError_t e = cudaFuncSetAttribute(
-              kern_flat, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_rows));
-          if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(dense_rows)");
-        }
-        kern_flat<<<dim3(unsigned(want), 1u, unsigned(ngroups)), nt, smem_rows, ctx->stream>>>(
-            a, int(totL), cpr, nw / cpr * cpr, DC, a.rows * nbatch);
-        return check_cuda(ctx, cudaGetLastError(), "dense_rows_kernel");
-      }
       kern<<<dim3(unsigned(per_item), unsigned(nbatch), unsigned(ngroups)), nt, smem_rows,
-             ctx->stream>>>(a, int(totL), cpr, used, DC, 0);
+             ctx->stream>>>(a, int(totL), cpr, used, DC);
       return check_cuda(ctx, cudaGetLastError(), "dense_rows_kernel");
     };
     const bool fine = int64_t(cpr) * 256 * 5 > a.L * 6;
     auto rows_for = [&](auto nl) -> int {
       constexpr int NL = decltype(nl)::value;
-      return fine ? launch_rows(dense_rows_kernel<768, NL, false, true>,
-                                dense_rows_kernel<768, NL, true, true>, 768)
-                  : launch_rows(dense_rows_kernel<768, NL, false, false>,
-                                dense_rows_kernel<768, NL, true, false>, 768);
+      return fine ? launch_rows(dense_rows_kernel<768, NL, true>, 768)
+                  : launch_rows(dense_rows_kernel<768, NL, false>, 768);
     };
     switch (N - 1) {
       case 0:
