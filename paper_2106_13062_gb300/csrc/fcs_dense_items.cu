@@ -13,8 +13,13 @@
 // to two int32 bins, its lower 15 bits to one and the rest to the other, which
 // at most 2^15 entries cannot overflow.  Where that rounding, q / sqrt(12),
 // exceeds 1e-7 of the entries' geometric mean (which a few outliers hardly
-// move; N(0,1) entries are 20 times below), or an entry is not finite, the
-// block adds in FP32 with compare-and-swap atomics instead.
+// move; N(0,1) entries are 20 times below), one int32 bin takes the entries as
+// multiples of 2^(E - 17) and the other, in FP32 with compare-and-swap
+// atomics, what that leaves of them, so that large entries cost the small ones
+// no digits (200 tensors of 64 x 64 with log-normal entries, D = 5: error 2.6e-8
+// for 1.1e-7 with FP32 sums alone, 49 us for 43).
+// Entries that are not finite, or too large or small for the powers of two, are
+// added in FP32 as they are.
 #include <algorithm>
 
 #include "fcs_dense_items.cuh"
@@ -23,7 +28,7 @@ namespace fcs {
 namespace {
 
 constexpr int kNT = 256;
-constexpr int kMaxEntries = 8192;         // per tensor; 2^15 would still be exact
+constexpr int kMaxEntries = 8192;         // per tensor
 
 struct ItemArgs {
   int N, D, n, tot, Jt;
@@ -46,7 +51,7 @@ __global__ void __launch_bounds__(kNT) dense_items_kernel(ItemArgs a) {
   int *lb = hb + a.D * a.Jt;                               // [D][Jt]
   int *tab = lb + a.D * a.Jt;                              // [D][tot] hash << 1 | negative, -1
   uint16_t *bin = reinterpret_cast<uint16_t *>(tab + a.D * a.tot);   // [D][n] bin << 1 | negative
-  float *fb = reinterpret_cast<float *>(hb);
+  float *lf = reinterpret_cast<float *>(lb);
   __shared__ float red[kNT / 32];
   __shared__ int exps[kNT / 32], nonzero[kNT / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -117,7 +122,11 @@ __global__ void __launch_bounds__(kNT) dense_items_kernel(ItemArgs a) {
     // log2 of both sides of q / sqrt(12) <= 1e-7 * geometric mean
     const bool fixed = finite && nz > 0 && E > -120 && E < 95 &&
                        float(E) - 1.8f <= float(ex) / float(nz) - 127.f - 23.3f;
-    const float q = fixed ? ldexpf(1.f, E) : 1.f, inv_q = fixed ? ldexpf(1.f, -E) : 1.f;
+    // otherwise the two parts of every entry, or no integers at all
+    const bool parts = !fixed && finite && nz > 0 && E > -120 && E < 95;
+    if (parts) E += 13;
+    const float q = fixed || parts ? ldexpf(1.f, E) : 1.f;
+    const float inv_q = fixed || parts ? ldexpf(1.f, -E) : 1.f;
     for (int e = tid; e < a.n; e += kNT) {
       const float x = __ldg(T + e);
       if (fixed) {
@@ -130,9 +139,14 @@ __global__ void __launch_bounds__(kNT) dense_items_kernel(ItemArgs a) {
           atomicAdd(&lb[d * a.Jt + (t >> 1)], v & 0x7fff);
         }
       } else {
+        // (|xi| <= 2^17: 2^13 entries of a bin stay below 2^31; r is exact)
+        const int xi = parts ? __float2int_rn(x * inv_q) : 0;
+        const float r = parts ? fmaf(-q, float(xi), x) : x;
         for (int d = 0; d < a.D; ++d) {
           const unsigned t = bin[d * a.n + e];
-          if (t != 0xffffu) atomicAdd(&fb[d * a.Jt + (t >> 1)], (t & 1) ? -x : x);
+          if (t == 0xffffu) continue;
+          if (xi) atomicAdd(&hb[d * a.Jt + (t >> 1)], (t & 1) ? -xi : xi);
+          if (r != 0.f) atomicAdd(&lf[d * a.Jt + (t >> 1)], (t & 1) ? -r : r);
         }
       }
     }
@@ -140,7 +154,9 @@ __global__ void __launch_bounds__(kNT) dense_items_kernel(ItemArgs a) {
     float *out = a.out + item * a.obs;
     for (int e = tid; e < a.D * a.Jt; e += kNT) {
       // (a 46-bit integer is exact in FP64; q is a power of two)
-      out[e] = fixed ? float((double(hb[e]) * 32768. + double(lb[e])) * double(q)) : fb[e];
+      out[e] = fixed   ? float((double(hb[e]) * 32768. + double(lb[e])) * double(q))
+               : parts ? float(double(hb[e]) * double(q) + double(lf[e]))
+                       : lf[e];
       hb[e] = 0;
       lb[e] = 0;
     }
