@@ -352,8 +352,9 @@ __global__ void __launch_bounds__(NT) contract_kernel(ContractArgs a,
 // ---------------------------------------------------------------- P = 16384
 // contract_kernel on the row-pair engine: one CTA per (item b, sketch d), two
 // to an SM (contract_kernel's registers and buffers leave room for one).  The
-// running product is in tensor memory between transforms; every forward
-// transform leaves twice the spectrum, so results scale by 2^-transforms.
+// running product is in tensor memory between transforms, at the scale that it
+// has in contract_kernel: the spectra are halved on the way (the unpack leaves
+// twice the values), or a product of N would run out of range 2^N earlier.
 template <int NR>
 __global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
     contract_pair_kernel(ContractArgs a, const float2 *__restrict__ tw) {
@@ -427,7 +428,8 @@ __global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
     const bool dot = (all || both) && k == N - 1;
     if (k == (all ? N - 1 : 0)) spec_wait();         // first use of the spectrum
     if (w0) {
-      const float2 x = pfft::column0<NR>(B, t3);
+      float2 x = pfft::column0<NR>(B, t3);
+      x = make_float2(0.5f * x.x, 0.5f * x.y);
       if (dot) {
         const float2 y = all ? slot_mul(p0, x, lane == 0) : x;
         const float2 g = all ? f0 : p0;
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
 #pragma unroll 1
     for (int c = 0; c < Geo::NCP; ++c) {
       pfft::C2 xa[H], xc[H];
-      pfft::column_step<NR>(B, t2, c, xa, xc);
+      pfft::column_step<NR, true>(B, t2, c, xa, xc);
       pfft::unpack<NR>(t2, c, xa, xc);
       const uint32_t o = tp + uint32_t(c) * (8 * H);
       __syncwarp();                                  // tensor-memory accesses are warp-wide
@@ -487,7 +489,7 @@ __global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
     if (tid == 0) {
       float t = 0.f;
       for (int w = 0; w < NT / 32; ++w) t += red[w];
-      (all ? a.raw : a.raw_all)[b * a.D + d] = t / (float(2 * M) * float(1 << N));
+      (all ? a.raw : a.raw_all)[b * a.D + d] = t / float(2 * M);
     }
   }
   if (!all) {
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(pfft::Geo<NR>::NT, pfft::Geo<NR>::CTAS)
     const int8_t *sm = a.s + d * a.m.ldh + a.m.off[m];
     const int64_t Im = a.m.I[m];
     float *rawbd = a.raw + (b * a.D + d) * Im;
-    const float sc = 1.0f / (float(M) * float(1 << (N - 1)));
+    const float sc = 1.0f / float(M);
     for (int64_t i = tid; i < Im; i += NT) {
       const int pz = __ldg(hm + i);
       const float v = unsigned(pz) < unsigned(2 * M) ? Bf[pz] : __int_as_float(0x7fc00000);

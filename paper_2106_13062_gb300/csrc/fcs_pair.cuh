@@ -426,8 +426,9 @@ __device__ __forceinline__ void pair_powers(C2 *P, const float2 *w) {
 //   xc[0] = (C[0], C[H]), xc[K] = (C[K + H], C[K]) for K > 0,
 //   C[(q1 + 1) mod NR] = Z[512 - u + 512 q1]
 // (the second column's twiddles are the conjugates of the first's, which
-// rotates its DFT's output by one).
-template <int NR>
+// rotates its DFT's output by one).  HALF: all of it times 1/2, by the first
+// twiddles.
+template <int NR, bool HALF = false>
 __device__ __forceinline__ void column_step(const float4 *B, const float2 *t2, int c, C2 *xa,
                                             C2 *xc) {
   using G = Geo<NR>;
@@ -442,7 +443,8 @@ __device__ __forceinline__ void column_step(const float4 *B, const float2 *t2, i
 #pragma unroll
   for (int b = 0; b < G::LNR; ++b) w[b] = t2[b * 256 + t];
   C2 P[G::H];
-  P[0] = C2{pk(1.f, w[0].x), pk(0.f, w[0].y)};
+  constexpr float f = HALF ? 0.5f : 1.f;
+  P[0] = C2{pk(f, f * w[0].x), pk(0.f, f * w[0].y)};
   pair_powers<G::LNR>(P, w);
 #pragma unroll
   for (int k = 0; k < G::H; ++k) {
@@ -458,7 +460,8 @@ __device__ __forceinline__ void column_step(const float4 *B, const float2 *t2, i
 
 // Real-FFT unpack of the column pair, in place: xa[K] holds TWICE X[q] and
 // xc[(H - K) mod H] TWICE X[M - q] for q = u + 512 K (low half) and
-// u + 512 (K + H) (high half).
+// u + 512 (K + H) (high half); X[q] and X[M - q] themselves after a column
+// step with HALF.
 template <int NR>
 __device__ __forceinline__ void unpack(const float2 *t2, int c, C2 *xa, C2 *xc) {
   using G = Geo<NR>;
