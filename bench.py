@@ -677,7 +677,7 @@ class BatchWorkload:
             self.grain = self.plan.config()[0]
         else:
             self.grain = fcs.fcs_batch_autotune(ctx, probs)
-            self.plan = fcs.BatchPlan(ctx, probs, grain=self.grain)
+            self.plan = fcs.BatchPlan(ctx, probs)    # the tuned cut and class shapes
         self.plan.launch()
         torch.cuda.synchronize()
         self.graph = torch.cuda.CUDAGraph()

@@ -321,21 +321,24 @@ int fcs_batch_plan_create_cfg(fcs_ctx *ctx, int nprob, const fcs_cp_problem *hos
                               int grain, int ncfg, const fcs_batch_class_cfg *host_cfg,
                               fcs_batch_plan **plan);
 
-/* The grain (0: chosen problem by problem) and class shapes a plan was built
+/* The given or autotuned grain (0: neither) and class shapes a plan was built
  * with: *host_ncfg classes (the
  * first max_cfg of them copied to host_cfg, largest FFT first). */
 int fcs_batch_plan_config(const fcs_batch_plan *plan, int *host_grain, int max_cfg,
                           fcs_batch_class_cfg *host_cfg, int *host_ncfg);
 
 /* Autotuner: times the whole batch on the device.  First the grain (ranks
- * per item: 0, i.e. problem by problem, 1, 2, 4, ... up to 64 and 2R) with every class at its default
- * shape; then, class by class from the largest FFT, every engine (for
+ * per item: 1, 2, 4, ... up to 64 and 2R) with every class at its default
+ * shape, and whether ranks cut problem by problem are faster than all of
+ * these; then, class by class from the largest FFT, every engine (for
  * P = 8192), thread_mult and items_per_cta with the other classes at their
  * best so far, a shape replacing the current one only when at least 3 %
  * faster.  The winner is
  * kept for this batch shape (sorted (FFT length, N, D, R, max I_n) of every
  * problem) and used by later plans of the same shape created with grain 0;
- * the grain goes to *host_best_grain; when the environment variable
+ * the best grain goes to *host_best_grain (a plan created with it has that
+ * grain, one created with 0 the problem-by-problem cut where that was faster);
+ * when the environment variable
  * FCS_AUTOTUNE_CACHE names a file, the table is persisted there. */
 int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem *host_probs,
                        int *host_best_grain);

@@ -35,7 +35,8 @@
 #include "fcs_batch_kernels.cuh"
 
 struct fcs_batch_state {
-  // batch signature -> autotuned grain and class shapes
+  // batch signature -> autotuned grain and class shapes; a shape of log2 M = 0
+  // marks a batch that is faster with its ranks cut problem by problem
   std::map<uint64_t, std::pair<int, std::vector<fcs::ClassCfg>>> tuned;
   bool cache_loaded = false;
   std::set<fcs_batch_plan *> plans;   // live plans; detached when the context goes
@@ -51,7 +52,7 @@ struct fcs_batch_plan {
   std::vector<fcs_cp_problem> longp;   // problems with P > 16384: their own launches
   void *long_ws = nullptr;             // their scratch, owned by the plan (graph-safe)
   size_t long_bytes = 0;
-  int grain = 0;                       // ranks per item it was built with
+  int grain = 0;                       // the given or tuned ranks per item, 0 = neither
 };
 
 namespace fcs {
@@ -186,7 +187,7 @@ uint64_t batch_signature(int nprob, const std::vector<HostProb> &hp,
 }
 
 // Cache file: one line per batch signature, "sig grain L:ntm:ipc:eng ..."
-// (a missing engine field reads as 0).
+// (a missing engine field reads as 0; "0:0:0:1" marks a cut problem by problem).
 void load_cache(fcs_batch_state &st) {
   if (st.cache_loaded) return;
   st.cache_loaded = true;
@@ -463,10 +464,11 @@ int batch_issue(fcs_ctx *ctx, char *base, const BatchBuild &b) {
 
 namespace {
 
-// Build a plan: lay the batch out in plan-owned device memory and upload the
+// Build a plan (grain 0: cut problem by problem; `label`: the grain that
+// fcs_batch_plan_config names): lay the batch out in plan-owned device memory and upload the
 // descriptors.
 int plan_create(fcs_ctx *ctx, int nprob_all, const fcs_cp_problem *q_all, int grain,
-                fcs_batch_plan **out, const std::vector<ClassCfg> *cfg = nullptr) {
+                fcs_batch_plan **out, const std::vector<ClassCfg> *cfg, int label) {
   *out = nullptr;
   // problems the batch kernels do not run follow them, one after another;
   // P = 32768 joins those when the plan would not fit the budget otherwise
@@ -552,7 +554,7 @@ int plan_create(fcs_ctx *ctx, int nprob_all, const fcs_cp_problem *q_all, int gr
     plan->outs.emplace_back(q_all[k].out, sizeof(float) * size_t(q_all[k].D) * size_t(jt));
   }
   plan->build = bb;
-  plan->grain = grain;
+  plan->grain = label;
   ctx->plan_bytes += bb.total + plan->long_bytes;
   ctx->batch->plans.insert(plan);
   *out = plan;
@@ -587,6 +589,12 @@ void plan_free(fcs_batch_plan *plan) {
   if (plan->dev) cudaFree(plan->dev);
   if (plan->long_ws) cudaFree(plan->long_ws);
   delete plan;
+}
+
+bool cut_by_problem(const std::vector<ClassCfg> &cfg) {
+  for (const ClassCfg &c : cfg)
+    if (c.L == 0) return true;
+  return false;
 }
 
 // The autotuned entry of this batch shape, or null.
@@ -655,8 +663,9 @@ extern "C" int fcs_batch_plan_create(fcs_ctx *ctx, int nprob, const fcs_cp_probl
   DeviceGuard g(ctx->device);
   // the autotuned shape of this batch (grain and class shapes), if any
   const auto *t = tuned_entry(ctx, nprob, host_probs);
-  if (grain < 1) grain = t ? t->first : 0;
-  return plan_create(ctx, nprob, host_probs, grain, plan, t ? &t->second : nullptr);
+  const int label = grain >= 1 ? grain : t ? t->first : 0;
+  if (grain < 1) grain = t && !cut_by_problem(t->second) ? t->first : 0;
+  return plan_create(ctx, nprob, host_probs, grain, plan, t ? &t->second : nullptr, label);
 }
 
 extern "C" int fcs_batch_plan_create_cfg(fcs_ctx *ctx, int nprob,
@@ -692,7 +701,7 @@ extern "C" int fcs_batch_plan_create_cfg(fcs_ctx *ctx, int nprob,
   if (rc) return rc;
   DeviceGuard g(ctx->device);
   if (grain < 1) grain = 0;
-  return plan_create(ctx, nprob, host_probs, grain, plan, &cfg);
+  return plan_create(ctx, nprob, host_probs, grain, plan, &cfg, grain);
 }
 
 extern "C" int fcs_batch_plan_config(const fcs_batch_plan *plan, int *host_grain, int max_cfg,
@@ -763,25 +772,33 @@ extern "C" int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem 
   // the whole batch timed on the device for each candidate
   auto timed = [&](int grain, const std::vector<ClassCfg> &cfg, float *ms) -> int {
     fcs_batch_plan *plan = nullptr;
-    int r = plan_create(ctx, nprob, host_probs, grain, &plan, &cfg);
+    int r = plan_create(ctx, nprob, host_probs, grain, &plan, &cfg, grain);
     if (r) return r;
     r = time_plan(ctx, plan, e0, e1, 3, ms);
     plan_free(plan);
     return r;
   };
-  // 1. ranks per item (0: chosen problem by problem), every class at its
-  //    default shape
+  // 1. ranks per item, and whether those chosen problem by problem are faster,
+  //    every class at its default shape
   std::vector<ClassCfg> cfg;
   for (int L : sizes) cfg.push_back(ClassCfg{L, 1, 1, default_engine(L)});
-  int best = 0;
+  int best = 1;
   float best_ms = 1e30f;
-  for (int grain = 0; grain <= 64 && grain < 2 * rmax && rc == FCS_OK;
-       grain = grain ? 2 * grain : 1) {
+  for (int grain = 1; grain <= 64 && grain < 2 * rmax && rc == FCS_OK; grain *= 2) {
     float ms = 0.f;
     rc = timed(grain, cfg, &ms);
     if (rc == FCS_OK && ms < best_ms) {
       best_ms = ms;
       best = grain;
+    }
+  }
+  int cut = best;
+  if (rc == FCS_OK) {
+    float ms = 0.f;
+    rc = timed(0, cfg, &ms);
+    if (rc == FCS_OK && ms < best_ms) {
+      best_ms = ms;
+      cut = 0;
     }
   }
   // 2. per class, threads per transform and items per CTA, the other
@@ -806,7 +823,7 @@ extern "C" int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem 
         c->ntm = sh.second;
         c->ipc = ipc;
         float ms = 0.f;
-        rc = timed(best, cfg, &ms);
+        rc = timed(cut, cfg, &ms);
         if (rc) break;
         if (ms < 0.97f * best_ms) {              // a clear gain, not timing noise
           best_ms = ms;
@@ -820,6 +837,7 @@ extern "C" int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem 
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc) return rc;
+  if (cut == 0) cfg.push_back(ClassCfg{0, 0, 0, 1});
   ctx->batch->tuned[batch_signature(nprob, hp, host_probs)] = {best, cfg};
   save_cache(*ctx->batch);
   if (host_best_grain) *host_best_grain = best;
