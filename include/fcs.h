@@ -334,12 +334,13 @@ int fcs_batch_plan_config(const fcs_batch_plan *plan, int *host_grain, int max_c
  * P = 8192), thread_mult and items_per_cta with the other classes at their
  * best so far, a shape replacing the current one only when at least 3 %
  * faster.  The winner is
- * kept for this batch shape (sorted (FFT length, N, D, R, max I_n) of every
- * problem) and used by later plans of the same shape created with grain 0;
+ * kept for this batch shape (sorted (FFT length, N, D, R, max I_n, and whether
+ * the longest J_n changes the launch) of every problem) and used by later plans of the same shape created with grain 0;
  * the best grain goes to *host_best_grain (a plan created with it has that
  * grain, one created with 0 the problem-by-problem cut where that was faster);
  * when the environment variable
- * FCS_AUTOTUNE_CACHE names a file, the table is persisted there. */
+ * FCS_AUTOTUNE_CACHE names a file, the table is persisted there (entries that
+ * kernels of another version were timed for stay in the file, unused). */
 int fcs_batch_autotune(fcs_ctx *ctx, int nprob, const fcs_cp_problem *host_probs,
                        int *host_best_grain);
 

@@ -167,11 +167,14 @@ int check_problem(fcs_ctx *ctx, int k, const fcs_cp_problem &q, HostProb *hp) {
   return FCS_OK;
 }
 
+// What a tuned shape is kept under: everything of the problems that decides
+// their launches, and the version of the kernels that it was timed with.
+constexpr uint64_t kTuneVersion = 2;
 uint64_t batch_signature(int nprob, const std::vector<HostProb> &hp,
                          const fcs_cp_problem *q) {
-  std::vector<std::array<int64_t, 5>> keys(nprob);
+  std::vector<std::array<int64_t, 6>> keys(nprob);
   for (int k = 0; k < nprob; ++k)
-    keys[k] = {hp[k].L, q[k].N, q[k].D, hp[k].R, hp[k].Imax};
+    keys[k] = {hp[k].L, q[k].N, q[k].D, hp[k].R, hp[k].Imax, hp[k].tall + 2 * int(hp[k].longp)};
   std::sort(keys.begin(), keys.end());
   uint64_t x = 1469598103934665603ull;   // FNV-1a
   auto mixin = [&](uint64_t v) {
@@ -180,6 +183,7 @@ uint64_t batch_signature(int nprob, const std::vector<HostProb> &hp,
       x *= 1099511628211ull;
     }
   };
+  mixin(kTuneVersion);
   mixin(uint64_t(nprob));
   for (auto &k : keys)
     for (int64_t v : k) mixin(uint64_t(v));

@@ -52,3 +52,48 @@ def test_returned_grain(fcs, monkeypatch, tmp_path):
         plan.close()
     c2.close()
     c.close()
+
+
+def test_hash_ranges_are_part_of_the_shape(fcs):
+    """P = 16384 with hash ranges that leave room for two resident blocks per
+    SM and with one that does not; P = 32768 on and off the batch kernels: a
+    shape tuned for one is not used for the other."""
+    c = fcs.Context()
+    for Ja, Jb in (([6500, 6500], [9000, 4000]), ([9000, 9000], [18000, 900])):
+        I, R, D = [120, 90], 6, 2
+        pa, _ka = _batch(fcs, c, [(I, Ja, R, D)], 911)
+        pb, _kb = _batch(fcs, c, [(I, Jb, R, D)], 912)
+        g = fcs.fcs_batch_autotune(c, pa)
+        for probs, grain in ((pa, g), (pb, 0)):
+            plan = fcs.BatchPlan(c, probs)
+            assert plan.config()[0] == grain
+            plan.close()
+    c.close()
+
+
+def _fnv(values):
+    x = 1469598103934665603
+    for v in values:
+        for b in range(8):
+            x = ((x ^ ((v >> (8 * b)) & 0xff)) * 1099511628211) & (2 ** 64 - 1)
+    return x
+
+
+def test_entries_of_earlier_kernels_are_not_used(fcs, monkeypatch, tmp_path):
+    """A file written before the engines changed (the signature was the hash
+    of the problem count and of (log2 M, N, D, R, max I_n)): read and kept,
+    but its grain is not taken."""
+    I, J, R, D = [120, 90], [6500, 6500], 6, 2
+    path = tmp_path / "tune.txt"
+    line = "%016x 4 13:1:2:1" % _fnv([1, 13, 2, D, R, max(I)])
+    path.write_text(line + "\n")
+    monkeypatch.setenv("FCS_AUTOTUNE_CACHE", str(path))
+    c = fcs.Context()
+    probs, _keep = _batch(fcs, c, [(I, J, R, D)], 921)
+    plan = fcs.BatchPlan(c, probs)
+    grain, cls = plan.config()
+    assert grain == 0 and [(P, ipc) for P, _, ipc, _, _ in cls] == [(16384, 1)]
+    plan.close()
+    fcs.fcs_batch_autotune(c, probs)
+    assert line in path.read_text().splitlines() and len(path.read_text().splitlines()) == 2
+    c.close()
