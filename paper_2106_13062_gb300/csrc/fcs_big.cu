@@ -120,8 +120,7 @@ int big_fft(fcs_ctx *ctx, const Pass1Args &a0, int64_t T, float2 *work) {
   Pass1Args a = a0;
   a.dst = work;
   const size_t smem = sizeof(float2) * padded_len(kM2);
-  cudaError_t e = cudaFuncSetAttribute(pass1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(smem));
+  const cudaError_t e = allow_smem(reinterpret_cast<const void *>(pass1_kernel), smem);
   if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(pass1)");
   for (int64_t t0 = 0; t0 < T; t0 += 65535) {
     const int64_t nt = std::min<int64_t>(65535, T - t0);
@@ -720,8 +719,7 @@ int big_sketch_cp(fcs_ctx *ctx, const Modes &m, int64_t R, int D, const float *c
                           "cudaMemsetAsync(G)");
       if (rc) return rc;
       const size_t smem = sizeof(float2) * padded_len(kM2);
-      cudaError_t e = cudaFuncSetAttribute(cp15_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           int(smem));
+      const cudaError_t e = allow_smem(reinterpret_cast<const void *>(cp15_kernel), smem);
       if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(cp15)");
       cp15_kernel<<<unsigned(f.ctas), kNT1, smem, ctx->stream>>>(a, ctx->twiddle);
       return check_cuda(ctx, cudaGetLastError(), "cp15_kernel");

@@ -624,10 +624,8 @@ int launch_contract(fcs_ctx *ctx, ContractArgs &a, int64_t Jt, bool need_spec,
   const size_t smem2 = FftSmem<LOG2M>::bytes(a.sb);
   auto k1 = spectrum_kernel<LOG2M, NT>;
   auto k2 = contract_kernel<LOG2M, NT>;
-  cudaError_t e = cudaSuccess;
-  if (smem1 > 48 * 1024) e = allow_smem(reinterpret_cast<const void *>(k1), smem1);
-  if (e == cudaSuccess && smem2 > 48 * 1024)
-    e = allow_smem(reinterpret_cast<const void *>(k2), smem2);
+  cudaError_t e = allow_smem(reinterpret_cast<const void *>(k1), smem1);
+  if (e == cudaSuccess) e = allow_smem(reinterpret_cast<const void *>(k2), smem2);
   if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(contract)");
   if (need_spec) {
     k1<<<a.D, NT, smem1, ctx->stream>>>(a.fcsT, Jt, Jt, sb_spec, a.spec, ctx->twiddle);

@@ -699,11 +699,8 @@ extern "C" int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
   const int threads = 1024;
   auto launch = [&](auto kern) -> int {
     const size_t sm = use_smem ? smem : 0;
-    if (sm > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           int(sm));
-      if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(dense)");
-    }
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), sm);
+    if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(dense)");
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sm);
     if (per_sm < 1) per_sm = 1;
@@ -730,11 +727,8 @@ extern "C" int fcs_sketch_dense(fcs_ctx *ctx, int N, const int64_t *host_I,
   if (vec && a.m.J[N - 1] <= 32767 && smem_rows <= 200 * 1024 && a.rows < (int64_t(1) << 31)) {
     const int cpr = cpr_rows;
     auto launch_rows = [&](auto kern, int nt) -> int {
-      if (smem_rows > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(smem_rows));
-        if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(dense_rows)");
-      }
+      const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), smem_rows);
+      if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(dense_rows)");
       int per_sm = 1;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem_rows);
       if (per_sm < 1) per_sm = 1;

@@ -207,10 +207,8 @@ int dense_items(fcs_ctx *ctx, int N, const int64_t *I, const int64_t *stride, co
   a.h = h;
   a.s = s;
   a.out = out;
-  const void *kern = reinterpret_cast<const void *>(dense_items_kernel);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) !=
-      cudaSuccess)
-    return check_cuda(ctx, cudaGetLastError(), "cudaFuncSetAttribute(dense_items)");
+  const cudaError_t e = allow_smem(reinterpret_cast<const void *>(dense_items_kernel), smem);
+  if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(dense_items)");
   const int per_sm = std::max(1, std::min(8, int(size_t(233472) / (smem + 2048))));
   const int64_t blocks = std::min<int64_t>(nbatch, int64_t(ctx->sm_count) * per_sm);
   dense_items_kernel<<<unsigned(blocks), kNT, smem, ctx->stream>>>(a);

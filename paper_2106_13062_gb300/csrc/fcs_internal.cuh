@@ -92,9 +92,10 @@ struct DeviceGuard {
 // limit is always set to the same value, beyond which no kernel here goes: it
 // belongs to the kernel and not to a launch, so a smaller value set for one
 // launch would refuse another, larger one that was prepared before it.
+// (Without it the limit is 48 KiB less the kernel's static arrays.)
 constexpr size_t kMaxDynSmem = 232448 - 1024;      // 227 KiB less room for static arrays
 inline cudaError_t allow_smem(const void *kern, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
+  if (bytes <= 47 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               int(bytes > kMaxDynSmem ? bytes : kMaxDynSmem));
 }

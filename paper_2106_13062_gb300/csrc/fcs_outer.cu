@@ -107,11 +107,8 @@ int launch_outer(fcs_ctx *ctx, int64_t nbatch, int64_t L, int D, int64_t La, int
                  const float *fa, const float *fb, float *out, int mult) {
   const int sb = int(((La > Lb ? La : Lb) + 3) / 4 * 4);
   auto go = [&](auto kern, int nt, size_t smem) -> int {
-    if (smem > 48 * 1024) {
-      cudaError_t e =
-          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-      if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(outer)");
-    }
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), smem);
+    if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(outer)");
     kern<<<dim3(unsigned(D), unsigned(nbatch)), nt, smem, ctx->stream>>>(fa, fb, La, Lb, L, D, sb,
                                                                          out, ctx->twiddle);
     return check_cuda(ctx, cudaGetLastError(), "outer_kernel");

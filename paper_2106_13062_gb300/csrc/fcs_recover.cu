@@ -269,11 +269,8 @@ int launch_recover(fcs_ctx *ctx, RecoverArgs &a, int64_t nbatch) {
       const bool idx4 = a.m.N == 4 && (reinterpret_cast<uintptr_t>(a.idx) & 15) == 0 &&
                         (a.ibs % 4) == 0;
       auto pick = [&](auto kern) -> int {
-        if (sm2 > 48 * 1024) {
-          cudaError_t e =
-              cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm2));
-          if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(recover_simd)");
-        }
+        const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), sm2);
+        if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(recover_simd)");
         int per_sm = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 1024, sm2);
         if (per_sm < 1) per_sm = 1;
@@ -292,11 +289,8 @@ int launch_recover(fcs_ctx *ctx, RecoverArgs &a, int64_t nbatch) {
     }
     if (j16 && sm2 <= 220 * 1024 && a.tot < (1 << 30)) {
       auto kern = recover_smem_kernel<D>;
-      if (sm2 > 48 * 1024) {
-        cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm2));
-        if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(recover_smem)");
-      }
+      const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), sm2);
+      if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(recover_smem)");
       int per_sm = 1;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 512, sm2);
       if (per_sm < 1) per_sm = 1;
@@ -312,10 +306,8 @@ int launch_recover(fcs_ctx *ctx, RecoverArgs &a, int64_t nbatch) {
   const bool use_smem = smem <= 96 * 1024;
   auto kern = use_smem ? recover_kernel<D, true> : recover_kernel<D, false>;
   const size_t sm = use_smem ? smem : 0;
-  if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
-    if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(recover)");
-  }
+  const cudaError_t e = allow_smem(reinterpret_cast<const void *>(kern), sm);
+  if (e != cudaSuccess) return check_cuda(ctx, e, "cudaFuncSetAttribute(recover)");
   int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm);
   if (per_sm < 1) per_sm = 1;
