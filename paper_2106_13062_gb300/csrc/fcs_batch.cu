@@ -70,7 +70,10 @@ struct TransposeTask {
 // is the last one whose first tile is not beyond this one: every thread looks
 // at tasks of its own, so finding it costs one memory latency (a binary
 // search over 230 tasks costs eight, as long as the copy of a 32 x 32 tile).
-constexpr int kTI = 128;
+// kTI = 128 where that still makes a tile for every SM, 32 below, where a tile's
+// own time counts (plans of one order-3 problem of 300 x 1 to 300 x 64 at P = 4096:
+// 19.9 us with 128 rows and 18.1 with 32, of 1500 x 16, order 2, 27.2 and 25.4).
+template <int kTI>
 __global__ void __launch_bounds__(256) batch_transpose_kernel(const TransposeTask *__restrict__ tasks,
                                                               int ntasks) {
   __shared__ float tile[kTI][33];
@@ -359,7 +362,11 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
   float *ut_base = reinterpret_cast<float *>(g_base + g_bytes);
   std::vector<TransposeTask> tasks;
   size_t goff = 0, toff = 0, uoff = 0;
-  int64_t tiles = 0;
+  int64_t tiles = 0, tall_tiles = 0;
+  for (int k = 0; k < nprob; ++k)
+    for (int n = 0; n < q[k].N; ++n)
+      tall_tiles += ((q[k].I[n] + 127) / 128) * ((hp[k].R + 31) / 32);
+  const int ti = tall_tiles < ctx->sm_count ? 32 : 128;
   for (int k = 0; k < nprob; ++k) {
     BatchProb &P = probs[k];
     P.N = q[k].N;
@@ -392,7 +399,7 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
       T.I = q[k].I[n];
       T.R = P.R;
       T.ld = q[k].ldU[n];
-      T.tiles_i = (T.I + kTI - 1) / kTI;
+      T.tiles_i = (T.I + ti - 1) / ti;
       T.tile0 = tiles;
       tiles += T.tiles_i * ((T.R + 31) / 32);
       tasks.push_back(T);
@@ -427,6 +434,7 @@ int batch_build(fcs_ctx *ctx, int nprob, const fcs_cp_problem *q, int grain, cha
   memcpy(host_desc->data() + b_probs + b_items, tasks.data(),
          sizeof(TransposeTask) * tasks.size());
   bb.tiles = tiles;
+  bb.tile_rows = ti;
   *out = bb;
   return FCS_OK;
 }
@@ -436,7 +444,8 @@ int batch_issue(fcs_ctx *ctx, char *base, const BatchBuild &b) {
   int rc = check_cuda(ctx, cudaMemsetAsync(base + b.clear_off, 0, b.clear_bytes, ctx->stream),
                       "cudaMemsetAsync(batch accumulators)");
   if (rc) return rc;
-  batch_transpose_kernel<<<unsigned(b.tiles), dim3(32, 8), 0, ctx->stream>>>(
+  const auto transpose = b.tile_rows == 32 ? batch_transpose_kernel<32> : batch_transpose_kernel<128>;
+  transpose<<<unsigned(b.tiles), dim3(32, 8), 0, ctx->stream>>>(
       reinterpret_cast<const TransposeTask *>(base + b.tasks_off), b.ntasks);
   rc = check_cuda(ctx, cudaGetLastError(), "batch_transpose_kernel");
   if (rc) return rc;

@@ -35,6 +35,7 @@ struct BatchBuild {
   size_t clear_off = 0, clear_bytes = 0;
   int nitems = 0, ntasks = 0;
   int64_t tiles = 0;
+  int tile_rows = 0;         // of a tile of the factor transpose
   std::vector<BatchClass> classes;
 };
 
