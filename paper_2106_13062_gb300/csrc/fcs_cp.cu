@@ -256,11 +256,17 @@ int64_t pair_groups(int sm_count, int64_t R, int D, size_t smem) {
 // before it).
 template <int NR, class View>
 cudaError_t launch_pair(CpArgs &a, int sm_count, const float2 *tw, cudaStream_t st) {
-  const size_t smem = pfft::Smem<NR>::bytes((a.sb + 2 * NR - 1) / (2 * NR));
+  size_t smem = pfft::Smem<NR>::bytes((a.sb + 2 * NR - 1) / (2 * NR));
   const void *kern = reinterpret_cast<const void *>(cp_pair_kernel<NR, View>);
+  const int64_t groups = pair_groups<NR>(sm_count, a.R, a.D, smem);
+  // Blocks that are placed while prep ends go to the SMs that are free first,
+  // two to an SM, though others stay empty.  With a block for every SM at most,
+  // each asks for half of an SM's shared memory, so that no two share one
+  // (order 3, I = 300, P = 16384: 34.3 us a call and so 25.5 at R = 19, D = 8, 30.5
+  // and 25.2 at R = 32, D = 4).
+  if (groups * a.D <= sm_count) smem = std::max(smem, size_t(233472) / 2);
   const cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  const int64_t groups = pair_groups<NR>(sm_count, a.R, a.D, smem);
   void *args[] = {&a, &tw};
   return launch_after_prep(st, kern, dim3(unsigned(groups * a.D)), dim3(pfft::Geo<NR>::NT), smem,
                            args);
