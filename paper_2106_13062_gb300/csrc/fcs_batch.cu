@@ -24,6 +24,7 @@
 // signature (in the context, and in the file named by FCS_AUTOTUNE_CACHE
 // when that variable is set).
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <array>
@@ -248,6 +249,24 @@ ClassCfg class_cfg(int L, const std::vector<ClassCfg> *cfg) {
   return c;
 }
 
+// Resident blocks per SM of a class kernel.
+int class_blocks_per_sm(const ClassKernel &ck) {
+  int n = ck.per_sm;
+  if (n == 0 && (!ck.fn || allow_smem(ck.fn, ck.smem) != cudaSuccess ||
+                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, ck.fn, ck.nt, ck.smem) !=
+                     cudaSuccess)) {
+    cudaGetLastError();
+    n = 1;
+  }
+  return n < 1 ? 1 : n;
+}
+
+// Ranks per item of a problem of rank R: `want`, evened out over its items.
+int64_t even_ranks(int64_t want, int64_t R) {
+  const int64_t groups = (R + std::max<int64_t>(want, 1) - 1) / std::max<int64_t>(want, 1);
+  return (R + groups - 1) / groups;
+}
+
 // Ranks per item, problem by problem, when the caller names no grain.  Every
 // item of an FFT-size class is to take about the same time, in transforms:
 // a quarter of what one resident block gets of the class, so that the last
@@ -256,39 +275,48 @@ ClassCfg class_cfg(int L, const std::vector<ClassCfg> *cfg) {
 // its spectrum cost about as much as one.  A class with less work than that
 // takes as many items as there are resident blocks.  (One grain for all,
 // about four items per SM, gave the 64-problem mix items of up to 64
-// transforms and 3.4 waves of them at P = 16384.)
+// transforms and 3.4 waves of them at P = 16384.)  A batch of P = 32768 alone,
+// where a block fills an SM, takes the length whose waves end first while that
+// is up to 32 transforms per SM (order 3, D = 5, R = 64: 160 items in two waves
+// took 114 us, 110 in one 90).
 std::vector<int64_t> balanced_ranks(fcs_ctx *ctx, const std::vector<HostProb> &hp, int nprob,
                                     const fcs_cp_problem *q, const std::vector<ClassCfg> *cfg) {
-  std::map<int, double> per_item;         // by launch: 2 L + tall
-  auto key = [&](int k) { return 2 * hp[k].L + hp[k].tall; };
-  for (int k = 0; k < nprob; ++k) per_item[key(k)] += double(q[k].D) * double(hp[k].R) * q[k].N;
-  for (auto &c : per_item) {
+  std::vector<int64_t> r(nprob);
+  std::map<int, std::vector<int>> classes;          // by launch: 2 L + tall
+  for (int k = 0; k < nprob; ++k) classes[2 * hp[k].L + hp[k].tall].push_back(k);
+  const double sms = std::max(1, ctx->sm_count);
+  for (const auto &c : classes) {
+    const int L = c.first / 2;
     int64_t Imax = 1;
     int sb = 4;
-    for (int k = 0; k < nprob; ++k)
-      if (key(k) == c.first) {
-        Imax = std::max(Imax, hp[k].Imax);
-        sb = std::max(sb, hp[k].sb);
-      }
-    const ClassCfg cc = class_cfg(c.first / 2, cfg);
-    const ClassKernel ck = class_kernel(c.first / 2, cc.eng, cc.ntm, cc.ipc, Imax, sb);
-    int per_sm = ck.per_sm;
-    if (per_sm == 0 &&
-        (!ck.fn || allow_smem(ck.fn, ck.smem) != cudaSuccess ||
-         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ck.fn, ck.nt, ck.smem) !=
-             cudaSuccess)) {
-      cudaGetLastError();
-      per_sm = 1;
+    double total = 0.;
+    for (int k : c.second) {
+      Imax = std::max(Imax, hp[k].Imax);
+      sb = std::max(sb, hp[k].sb);
+      total += double(q[k].D) * double(hp[k].R) * q[k].N;
     }
-    if (per_sm < 1) per_sm = 1;
-    const double each = c.second / (double(std::max(1, ctx->sm_count)) * per_sm);
-    c.second = each <= 8. ? each : std::max(8., each / 4.);
-  }
-  std::vector<int64_t> r(nprob);
-  for (int k = 0; k < nprob; ++k) {
-    const int64_t want = std::max<int64_t>(1, int64_t(per_item[key(k)] / q[k].N + 0.5));
-    const int64_t groups = (hp[k].R + want - 1) / want;
-    r[k] = (hp[k].R + groups - 1) / groups;
+    const ClassCfg cc = class_cfg(L, cfg);
+    const int per_sm = class_blocks_per_sm(class_kernel(L, cc.eng, cc.ntm, cc.ipc, Imax, sb));
+    const double each = total / (sms * per_sm);
+    double len = each <= 8. ? each : std::max(8., each / 4.), half = 0.5;
+    if (L == 14 && classes.size() == 1 && each <= 32.) {
+      double least = 1e300;
+      for (int t = 1; t <= 40; ++t) {
+        int64_t items = 0, longest = 1;
+        for (int k : c.second) {
+          const int64_t rk = even_ranks(t / q[k].N, hp[k].R);
+          items += q[k].D * ((hp[k].R + rk - 1) / rk);
+          longest = std::max<int64_t>(longest, rk * q[k].N);
+        }
+        const double cost = (double(longest) + 1.) * std::ceil(double(items) / sms);
+        if (cost < least) {
+          least = cost;
+          len = t;
+        }
+      }
+      half = 0.;
+    }
+    for (int k : c.second) r[k] = even_ranks(int64_t(len / q[k].N + half), hp[k].R);
   }
   return r;
 }
