@@ -503,6 +503,18 @@ int batch_issue(fcs_ctx *ctx, char *base, const BatchBuild &b) {
   return FCS_OK;
 }
 
+int batch_round_grain(const fcs_ctx *ctx, int nprob, const fcs_cp_problem *q) {
+  int64_t work = 0, rmax = 1;
+  for (int k = 0; k < nprob; ++k) {
+    work += int64_t(q[k].D) * q[k].R;
+    rmax = std::max<int64_t>(rmax, q[k].R);
+  }
+  const int64_t g = work / (4 * int64_t(std::max(1, ctx->sm_count)));
+  int grain = 1;
+  while (grain * 2 <= g && grain < 64) grain *= 2;
+  return int(std::min<int64_t>(grain, rmax));
+}
+
 namespace {
 
 // Build a plan (grain 0: cut problem by problem; `label`: the grain that

@@ -276,8 +276,8 @@ std::vector<Req *> admit(fcs_server *S) {
     }
     if (S->inflight >= S->cfg.max_inflight) break;
     if (q->r.kind == FCS_REQ_CP && ncp >= S->cfg.max_batch) break;
-    // a CP request with P > 16384 (multi-kernel long-FFT route) gets a round
-    // of its own, so it does not hold back the completion of short requests
+    // a CP request with P > 16384 gets a round of its own, so it does not hold
+    // back the completion of short requests
     const bool longq = q->r.kind == FCS_REQ_CP && q->Jt > (int64_t(1) << fcs::kMaxLog2P);
     if (longq && !got.empty()) break;
     size_t doff = 0, poff = 0, koff = 0;
@@ -382,7 +382,7 @@ int issue_round(fcs_server *S, int si, std::vector<Req *> &reqs, Round &rd) {
       p.ldh = 0;
       p.out = q->dout;
       if (q->Jt > (int64_t(1) << fcs::kMaxLog2P)) {
-        // too long for the batch kernels: its own (multi-kernel) launch
+        // alone in its round: launches of its own
         rc = fcs_sketch_cp(ctx, p.N, p.I, p.J, p.R, p.D, p.U, p.ldU, p.lambda, p.h, p.s, p.ldh,
                            p.out);
         if (rc) return rc;
@@ -407,7 +407,7 @@ int issue_round(fcs_server *S, int si, std::vector<Req *> &reqs, Round &rd) {
   }
   // one batched launch for every CP request of the round
   if (!probs.empty()) {
-    const int grain = 0;
+    const int grain = fcs::batch_round_grain(ctx, int(probs.size()), probs.data());
     fcs::BatchBuild bb{};
     std::vector<char> desc;
     int rc = fcs::batch_build(ctx, int(probs.size()), probs.data(), grain, nullptr, &desc, &bb);
