@@ -18,6 +18,7 @@
 // for the duration of the call (fcs_contract's cache), so the power
 // iterations and sweeps transform each sketch once.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "fcs_div.cuh"
@@ -136,7 +137,8 @@ __global__ void __launch_bounds__(1024) als_gram_kernel(AlsArgs a) {
 // rows by one thread each, the factorisation by one thread and the solve's
 // vector in local memory; now 20 us): a warp factors, lane i holding row i, and
 // RM >= R lanes solve eight columns at a time, one element of each per lane (the
-// rows past R are those of the identity).
+// rows past R are those of the identity), again with a look at infinities where
+// something is not finite (looking at every quotient cost 2 us an update).
 constexpr int kUpdNT = 512;
 template <int RM>
 __global__ void __launch_bounds__(kUpdNT) als_update_kernel(AlsArgs a) {
@@ -198,27 +200,34 @@ __global__ void __launch_bounds__(kUpdNT) als_update_kernel(AlsArgs a) {
   float ss = 0.f;
   for (int64_t i0 = int64_t(tid / RM) * Q; i0 - int64_t(tid / RM) * Q < Im; i0 += GROUPS * Q) {
     float x[Q];
+    auto solve = [&](auto inf) {
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
-      x[q] = r < R && i0 + q < Im ? a.Mt[int64_t(r) * Im + i0 + q] : 0.f;
+      for (int q = 0; q < Q; ++q)
+        x[q] = r < R && i0 + q < Im ? a.Mt[int64_t(r) * Im + i0 + q] : 0.f;
 #pragma unroll
-    for (int j = 0; j < RM; ++j) {            // L y = b
+      for (int j = 0; j < RM; ++j) {            // L y = b
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const float y = quotient(x[q], dg, iv);
-        const float t = __shfl_sync(0xffffffffu, y, j, RM);
-        x[q] = r == j ? y : r > j ? x[q] - row[j] * t : x[q];
+        for (int q = 0; q < Q; ++q) {
+          const float y = quotient<decltype(inf)::value>(x[q], dg, iv);
+          const float t = __shfl_sync(0xffffffffu, y, j, RM);
+          x[q] = r == j ? y : r > j ? x[q] - row[j] * t : x[q];
+        }
       }
-    }
 #pragma unroll
-    for (int j = RM - 1; j >= 0; --j) {       // L^T x = y
+      for (int j = RM - 1; j >= 0; --j) {       // L^T x = y
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const float y = quotient(x[q], dg, iv);
-        const float t = __shfl_sync(0xffffffffu, y, j, RM);
-        x[q] = r == j ? y : r < j ? x[q] - colm[j] * t : x[q];
+        for (int q = 0; q < Q; ++q) {
+          const float y = quotient<decltype(inf)::value>(x[q], dg, iv);
+          const float t = __shfl_sync(0xffffffffu, y, j, RM);
+          x[q] = r == j ? y : r < j ? x[q] - colm[j] * t : x[q];
+        }
       }
-    }
+    };
+    solve(std::false_type());
+    bool finite = true;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) finite = finite && fabsf(x[q]) <= 3.402823466e38f;
+    if (!__all_sync(0xffffffffu, finite)) solve(std::true_type());
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       ss = fmaf(x[q], x[q], ss);
