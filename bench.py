@@ -245,7 +245,8 @@ class CpWorkload:
         sm_mhz = float(measured_peaks().get("sm_max_mhz", 2070.0))
         peak = props.multi_processor_count * 128 * 2 * sm_mhz * 1e6 / 1e12
         ach = self.flops() / (t / 1e3) / 1e12
-        files = ["fcs_cp.cu", "fcs_cp_run.cuh", "fcs_pair.cuh", "fcs_fft.cuh", "fcs_hash.cuh", "fcs_internal.cuh"]
+        files = ["fcs_cp.cu", "fcs_cp_run.cuh", "fcs_dit.cuh", "fcs_pair.cuh", "fcs_fft.cuh",
+                 "fcs_hash.cuh", "fcs_internal.cuh"]
         return {"kernel": "cp_pair_kernel (fcs_sketch_cp_seeded: prep launch with the hash "
                           "tables + fused sketch)",
                 "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
@@ -743,12 +744,13 @@ class BatchWorkload:
                                             ["fcs_batch.cu", "fcs_batch_kernels.cuh",
                                              "fcs_batch_k0.cu", "fcs_batch_k1.cu",
                                              "fcs_batch_k2.cu", "fcs_batch_k3.cu",
-                                             "fcs_batch_k4.cu", "fcs_cp_run.cuh", "fcs_pair.cuh",
+                                             "fcs_batch_k4.cu", "fcs_cp_run.cuh", "fcs_dit.cuh",
+                                             "fcs_pair.cuh",
                                              "fcs_fft.cuh", "fcs_internal.cuh"]),
                 "peak_source": f"derived: {props.multi_processor_count} SMs x 128 FP32 lanes "
                                f"x 2 flop/FMA x {sm_mhz:.0f} MHz",
                 "avg_launch_ms": t, "grain": self.grain,
-                "classes": [{"fft_len": P, "engine": "row-pair" if e else "slot FFT",
+                "classes": [{"fft_len": P, "engine": ("warp-DIT" if P == 8192 else "row-pair") if e else "slot FFT",
                              "thread_mult": m, "items_per_cta": i, "threads": n}
                             for P, m, i, n, e in self.plan.config()[1]],
                 "plain_per_problem_ms": plain_ms,

@@ -228,8 +228,9 @@ def exported_symbols():
 # A small call is bound by the time these take on the host, so each reads an
 # attribute of a tensor once, reads the current stream without a Stream object,
 # and makes names for error texts only for an error.  Back-to-back calls, us
-# before and after: 20 x 20 x 20 sketch from a seed 38.9 and 30.6, a ragged one of
-# order 3 49.1 and 38.8, tensor regression layer (two calls) 39.7 and 28.7.
+# before and after, medians over several machines whose host parts differ by 20 %:
+# 20 x 20 x 20 sketch from a seed 38 and 32.5; tensor regression layer (two calls)
+# 39.7 and 28.7 on one.
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 

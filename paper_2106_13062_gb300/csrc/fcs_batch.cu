@@ -50,7 +50,7 @@ struct fcs_batch_plan {
   fcs::BatchBuild build{};
   fcs_ctx *owner = nullptr;
   std::vector<std::pair<const void *, size_t>> outs;   // output sketches written
-  std::vector<fcs_cp_problem> longp;   // problems with P > 16384: their own launches
+  std::vector<fcs_cp_problem> longp;   // problems outside the chain: their own launches
   void *long_ws = nullptr;             // their scratch, owned by the plan (graph-safe)
   size_t long_bytes = 0;
   int grain = 0;                       // the given or tuned ranks per item, 0 = neither
